@@ -238,13 +238,24 @@ def _outputs(sizes, dev, costs, second=False):
     return flat, outs
 
 
+_stream = []
+
+
+def _shared_stream():
+    """One stream for every context of the no-allocation call: its calls share one scratch array and have to be
+    serialised by the caller."""
+    if not _stream:
+        _stream.append(torch.cuda.Stream(device=0))
+    return _stream[0]
+
+
 def prepare(case, seed):
     dev = torch.device("cuda", 0)
     gen = torch.Generator(device=dev)
     gen.manual_seed(seed * 7919 + 17)
     prm = configs.MatchParams(n_scales=case["levels"], iters=case["iters"], eps=case["eps"], cost=case["cost"],
                               sub_scales=case["sub_scales"])
-    M = ff.Matcher(prm, 0)
+    M = ff.Matcher(prm, 0, _shared_stream() if case["op"] == "noalloc" else None)
     if case["table"]:
         with open(_TABLE) as f:
             for level, cfg in enumerate(json.load(f)["kitti_1242x375"]):
