@@ -310,14 +310,35 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
     return true;
 }
 
-// Default propagation configuration of a level when it has not been tuned: large tiles with one iteration per
-// launch when the level fills the GPU, otherwise small tiles with fused iterations (idle SMs absorb the halo).
-TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T) {
+// Default propagation configuration of a pass that has not been tuned, by its pixels (all problems of its launches):
+// from 20,000 pixels the queue variant of the dataflow form (every iteration in one launch, no resident grid needed),
+// in tiles small enough to keep every SM busy; below, where a pass is a chain of half-sweeps on a few SMs, the tile
+// form with two iterations per launch, whose halo idle SMs absorb.  The lines are the near-best of a sweep over single
+// pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both costs.  Levels 0 to 4 of the
+// 1242x375 pair (us): 661, 236, 115, 85 and 69 instead of 844, 375, 294, 113 and 75 with the rule for the tile form
+// below; of the 1920x1080 pair 2800, 713, 258, 119 and 83 instead of 3280, 935, 594, 475 and 142.
+TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow_ok) {
+    if (dataflow_ok) {
+        if (level_pix_all > 800000) return {48, 24, 1, 128, 0, 0, 1};
+        if (level_pix_all > 450000) return {56, 24, 1, 256, 0, 0, 1};
+        if (level_pix_all > 300000) return {32, 32, 1, 256, 0, 0, 1};
+        if (level_pix_all > 200000) return {24, 24, 1, 256, 0, 0, 1};
+        if (level_pix_all > 130000) return {24, 16, 1, 256, 0, 0, 1};
+        if (level_pix_all > 75000) return {20, 12, 1, 256, 0, 0, 1};
+        if (level_pix_all > 50000) return {26, 16, 1, 512, 0, 0, 1};
+        if (level_pix_all > 20000) return {16, 8, 1, 256, 0, 0, 1};
+        if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
+        return {8, 8, std::min(2, T), 256, 0};
+    }
+    // tile form only (a launch per group of iterations): large tiles with one iteration per launch when the level
+    // fills the GPU, otherwise small tiles with fused iterations
     const int64_t slots = (int64_t)c->n_sms * 2;
     if (level_pix_all / (32 * 32) >= 2 * slots) return {32, 32, 1, 256, 0};
     if (level_pix_all / (32 * 16) >= 2 * slots) return {32, 16, 1, 256, 0};
-    if (level_pix_all / (16 * 16) >= slots) return {16, 16, std::min(2, T), 256, 1};
-    return {8, 8, std::min(3, T), 256, 1};
+    if (level_pix_all > 50000) return {16, 16, 1, 256, 0};
+    if (level_pix_all > 20000) return {16, 8, 1, 256, 0};
+    if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
+    return {8, 8, std::min(2, T), 256, 0};
 }
 
 ff_status enqueue_launch(ff_ctx* c, const Launch& L) {
@@ -629,10 +650,10 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
             tc.k = std::min(tc.k, T);
         } else {
             auto it = c->tuned.find(TuneKey{pass, gdim(jobs[0].a->ws[s], k), gdim(jobs[0].a->hs[s], k), nj, T});
-            tc = it != c->tuned.end() ? it->second : default_cfg(c, level_pix, T);
+            tc = it != c->tuned.end() ? it->second : default_cfg(c, level_pix, T, true);
         }
         size_t cl_smem = 0;
-        if (tc.cluster > 0 && !cluster_fits(c, jobs, s, k, tc, &cl_smem)) tc = default_cfg(c, level_pix, T);
+        if (tc.cluster > 0 && !cluster_fits(c, jobs, s, k, tc, &cl_smem)) tc = default_cfg(c, level_pix, T, true);
         const bool cl = tc.cluster > 0, df = tc.dataflow > 0;
         if (df) tc.k = T;  // one launch, one iteration per tile task
         const size_t smem = cl ? 0 : prop_smem_bytes(tc.tw, tc.th, df ? 1 : tc.k);
@@ -1247,7 +1268,7 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
                 best_d = d;
             }
         }
-        tc = best ? *best : default_cfg(c, level_pix_all, T);
+        tc = best ? *best : default_cfg(c, level_pix_all, T, dataflow_ok);
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     if (tc.dataflow > 0) return {tc.tw, tc.th, T, tc.threads, 0, tc.dataflow};
