@@ -139,7 +139,7 @@ struct FineWht {
 };
 
 struct TileCfg {
-    int tw, th, k, threads, spec;  // tile interior, iterations fused per launch, CTA size, speculative random
+    int tw, th, k, threads, spec;  // tile interior, iterations fused per launch, CTA size (spec: without effect)
     int cluster = 0;               // > 0: the cluster form with this many CTAs per problem (tw, th unused)
     int dataflow = 0;              // 1: the dataflow form (every iteration in one launch; k unused), 2: affine
 };
@@ -149,12 +149,9 @@ const TileCfg kCands[] = {
     {64, 32, 1, 256, 0}, {32, 32, 1, 256, 0}, {32, 16, 1, 256, 0}, {16, 16, 1, 256, 0}, {32, 16, 2, 256, 0},
     {16, 16, 2, 256, 0}, {16, 8, 2, 256, 0},  {16, 8, 3, 256, 0},  {8, 8, 3, 256, 0},   {8, 8, 6, 256, 0},
     {32, 16, 1, 128, 0}, {16, 16, 1, 128, 0}, {16, 8, 2, 128, 0},  {8, 8, 3, 128, 0},   {32, 32, 1, 512, 0},
-    {32, 16, 2, 512, 0}, {16, 16, 2, 512, 0}, {24, 24, 1, 512, 0}, {32, 16, 1, 128, 1}, {16, 16, 1, 128, 1},
-    {16, 8, 2, 128, 1},  {8, 8, 3, 128, 1},   {32, 16, 1, 256, 1}, {16, 16, 1, 256, 1}, {16, 8, 2, 256, 1},
-    {8, 8, 3, 256, 1},   {32, 32, 1, 512, 1}, {16, 16, 2, 512, 1}, {24, 24, 1, 512, 1},
+    {32, 16, 2, 512, 0}, {16, 16, 2, 512, 0}, {24, 24, 1, 512, 0},
     // coarse levels: one pixel per thread per half-sweep (fewer dependent loads in a row)
-    {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},   {16, 16, 1, 512, 0}, {8, 8, 3, 512, 1},
-    {16, 8, 2, 512, 1},  {16, 16, 1, 512, 1}, {8, 8, 6, 512, 0},   {8, 8, 6, 512, 1},
+    {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},   {16, 16, 1, 512, 0}, {8, 8, 6, 512, 0},
     // fine levels: larger tiles recompute a smaller share of halo pixels
     {64, 32, 1, 128, 0}, {48, 32, 1, 128, 0}, {48, 32, 1, 256, 0}, {64, 16, 1, 128, 0}, {40, 24, 1, 128, 0},
     {48, 24, 1, 128, 0}, {64, 24, 1, 256, 0}, {64, 24, 1, 128, 0}, {96, 24, 1, 256, 0}, {80, 24, 1, 256, 0},
@@ -174,6 +171,11 @@ const TileCfg kCands[] = {
     {96, 32, 1, 512, 0, 0, 1},  {128, 32, 1, 512, 0, 0, 1}, {64, 64, 1, 512, 0, 0, 1},  {64, 27, 1, 512, 0, 0, 1},
     {32, 32, 1, 512, 0, 0, 1},  {26, 16, 1, 512, 0, 0, 1},  {16, 16, 1, 512, 0, 0, 1},  {16, 8, 1, 512, 0, 0, 1},
     {8, 8, 1, 512, 0, 0, 1},
+    // tiles whose regions (tile + 8) are a power of two wide, for the listed variant
+    {56, 16, 1, 256, 0, 0, 1},  {56, 20, 1, 256, 0, 0, 1},  {56, 24, 1, 256, 0, 0, 1},  {56, 32, 1, 256, 0, 0, 1},
+    {56, 40, 1, 256, 0, 0, 1},  {120, 24, 1, 256, 0, 0, 1}, {24, 12, 1, 256, 0, 0, 1},  {24, 16, 1, 256, 0, 0, 1},
+    {24, 24, 1, 256, 0, 0, 1},  {24, 40, 1, 256, 0, 0, 1},  {24, 16, 1, 128, 0, 0, 1},  {56, 32, 1, 512, 0, 0, 1},
+    {120, 40, 1, 512, 0, 0, 1},
     // its affine variant (fixed tiles per CTA, warm L1 across iterations): coarse levels, few tiles per CTA
     {26, 16, 1, 512, 0, 0, 2},  {32, 16, 1, 512, 0, 0, 2},  {16, 16, 1, 512, 0, 0, 2},  {16, 8, 1, 512, 0, 0, 2},
     {8, 8, 1, 512, 0, 0, 2},    {16, 8, 1, 256, 0, 0, 2},   {8, 8, 1, 256, 0, 0, 2},    {32, 16, 1, 256, 0, 0, 2},
@@ -304,7 +306,7 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
         if (!cluster_partition(w, h, t.cluster, bx, by)) return false;
         most = std::max(most, cluster_smem_bytes(w, h, bx, by));
     }
-    if (most > kMaxPropSmem || prop_cluster_capacity(t.cluster, t.threads, c->prm.cost, k > 0, most) < 1)
+    if (most > kMaxPropSmem || prop_cluster_capacity(t.cluster, t.threads, c->prm.cost, most) < 1)
         return false;
     *smem = most;
     return true;
@@ -314,14 +316,21 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
 // from 20,000 pixels the queue variant of the dataflow form (every iteration in one launch, no resident grid needed),
 // in tiles small enough to keep every SM busy; below, where a pass is a chain of half-sweeps on a few SMs, the tile
 // form with two iterations per launch, whose halo idle SMs absorb.  The lines are the near-best of a sweep over single
-// pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both costs.  Levels 0 to 4 of the
-// 1242x375 pair (us): 661, 236, 115, 85 and 69 instead of 844, 375, 294, 113 and 75 with the rule for the tile form
-// below; of the 1920x1080 pair 2800, 713, 258, 119 and 83 instead of 3280, 935, 594, 475 and 142.
+// pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both costs.  Passes the listed
+// variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the largest that leave the
+// queue more tiles than the 608 CTAs an SM's 2048 threads make (a Census distance is a third of the work, so larger
+// tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 567, 236, 115, 85 and 69 instead of 844, 375, 294, 113
+// and 75 with the rule for the tile form below; of the 1920x1080 pair 1816, 551, 258, 119 and 83 instead of 3280, 935,
+// 594, 475 and 142.
 TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow_ok) {
     if (dataflow_ok) {
-        if (level_pix_all > 800000) return {48, 24, 1, 128, 0, 0, 1};
-        if (level_pix_all > 450000) return {56, 24, 1, 256, 0, 0, 1};
-        if (level_pix_all > 300000) return {32, 32, 1, 256, 0, 0, 1};
+        if (prop_listed(level_pix_all, 56, 256, true)) {
+            const int64_t tiles = c->prm.cost == FF_COST_CENSUS ? 650 : 1000;
+            if (level_pix_all >= tiles * 56 * 40) return {56, 40, 1, 256, 0, 0, 1};
+            if (level_pix_all >= tiles * 56 * 24) return {56, 24, 1, 256, 0, 0, 1};
+            if (level_pix_all >= tiles * 56 * 16) return {56, 16, 1, 256, 0, 0, 1};
+            return {24, 16, 1, 256, 0, 0, 1};
+        }
         if (level_pix_all > 200000) return {24, 24, 1, 256, 0, 0, 1};
         if (level_pix_all > 130000) return {24, 16, 1, 256, 0, 0, 1};
         if (level_pix_all > 75000) return {20, 12, 1, 256, 0, 0, 1};
@@ -656,8 +665,10 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
         if (tc.cluster > 0 && !cluster_fits(c, jobs, s, k, tc, &cl_smem)) tc = default_cfg(c, level_pix, T, true);
         const bool cl = tc.cluster > 0, df = tc.dataflow > 0;
         if (df) tc.k = T;  // one launch, one iteration per tile task
-        const size_t smem = cl ? 0 : prop_smem_bytes(tc.tw, tc.th, df ? 1 : tc.k);
-        const int blocks = cl ? 0 : prop_blocks_per_sm(smem, tc.threads, tc.spec != 0, cost, k > 0, df) * c->n_sms;
+        const bool listed = !cl && prop_listed(level_pix, tc.tw, tc.threads, df);
+        if (listed) prop_fit_tile(tc.tw, tc.th);
+        const size_t smem = cl ? 0 : prop_launch_smem(tc.tw, tc.th, df ? 1 : tc.k, listed);
+        const int blocks = cl ? 0 : prop_blocks_per_sm(smem, tc.threads, cost, df, listed) * c->n_sms;
         for (int t0 = 0; t0 < T; t0 += tc.k) {
             int n_iter = std::min(tc.k, T - t0);
             bool last = t0 + n_iter == T;
@@ -672,7 +683,6 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
             l.prop.dataflow = df ? T : 0;
             l.prop.affine = tc.dataflow == 2;
             l.prop.threads = tc.threads;
-            l.prop.spec = tc.spec;
             l.prop.cost = cost;
             l.prop.grid = k > 0;
             l.prop.cluster = tc.cluster;
@@ -680,6 +690,7 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
             l.prop.wait_limit = c->wait_limit;
             l.prop.withhold = c->withhold;
             l.prop.err = c->d_err;
+            l.prop.listed = listed;
             size_t oq = queue.size();
             std::vector<int> pidx(nj), ntiles(nj);
             for (int j = 0; j < nj; j++) {
@@ -716,7 +727,8 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
                 pp.level = s + 8 * k;  // the hash stream of this level or grid
                 pp.dir = jobs[j].dir;
                 pp.seed = c->prm.seed;
-                pp.rs_radius = jobs[j].rs_radius;
+                pp.rs_radius = (uint16_t)jobs[j].rs_radius;
+                pp.T = (uint16_t)T;
                 pidx[j] = (int)props.size();
                 props.push_back(pp);
             }
@@ -1077,9 +1089,7 @@ void wave_shape(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k, 
     for (const DirJob& j : jobs)
         n += (int64_t)((grid_dim(j.a->ws[s], k) + t.tw - 1) / t.tw) * ((grid_dim(j.a->hs[s], k) + t.th - 1) / t.th);
     *tiles = n;
-    *slots = (int64_t)prop_blocks_per_sm(prop_smem_bytes(t.tw, t.th, t.k), t.threads, t.spec != 0, c->prm.cost,
-                                         k > 0) *
-             c->n_sms;
+    *slots = (int64_t)prop_blocks_per_sm(prop_smem_bytes(t.tw, t.th, t.k), t.threads, c->prm.cost, false, false) * c->n_sms;
 }
 
 // A launch whose last wave is a small remainder of tiles runs at about the speed of one more full wave.  The
@@ -1271,8 +1281,10 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
         tc = best ? *best : default_cfg(c, level_pix_all, T, dataflow_ok);
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
-    if (tc.dataflow > 0) return {tc.tw, tc.th, T, tc.threads, 0, tc.dataflow};
-    return {tc.tw, tc.th, std::min(tc.k, T), tc.threads, tc.spec, 0};
+    tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);
+    const bool listed = prop_listed(level_pix_all, tc.tw, tc.threads, tc.dataflow > 0);
+    if (listed) prop_fit_tile(tc.tw, tc.th);
+    return {tc.tw, tc.th, tc.k, tc.threads, listed, tc.dataflow};
 }
 
 int* ctx_err_word(ff_ctx* c) {

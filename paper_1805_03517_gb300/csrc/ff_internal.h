@@ -152,7 +152,8 @@ struct PropProblem {  // one (pair, direction, level) of a propagation launch
     int level;       // stream id of the random-search hash: the level, + 8 * log2(g) on a sub-scale grid
     int dir;
     uint32_t seed;
-    int rs_radius;
+    uint16_t rs_radius;
+    uint16_t T;      // iterations of the whole pass (its last one leaves plain costs, see the state word)
     // dataflow form only: the state buffers iterations alternate with (iteration t writes flow_alt for even t,
     // flow_in for odd t, flow_out for the last) and the tiles' progress counters (zero at the launch's start)
     uint32_t* flow_alt;
@@ -163,7 +164,6 @@ struct PropLaunch {
     int tw, th;      // tile interior
     int max_iter;    // largest n_iter of the launch (sizes the shared-memory halo)
     int threads;     // CTA size: 128, 256 or 512
-    int spec;        // 1: load the random candidate together with the neighbour candidates
     int cost;        // FF_COST_WHT_SAD or FF_COST_CENSUS
     int grid;        // 1: the problems are sub-scale grids (g > 1)
     int cluster;     // 0: tiles from a queue; n = 1..16: cluster form, one cluster of n CTAs per problem
@@ -174,12 +174,21 @@ struct PropLaunch {
     int withhold;    // test of the bounded waits: the cluster form sends no block edges, the dataflow form
                      // publishes no tile progress
     int* err;        // device error word (kErrClusterEdges / kErrDataflow when a wait gave up)
+    int listed;      // dataflow form: 1 = the listed variant (prop_listed), 0 = the direct one
 };
 constexpr int kErrClusterEdges = 3;  // error-word codes of expired waits (1, 2: tensor-core seed)
 constexpr int kErrDataflow = 4;
-constexpr size_t kMaxPropSmem = 200 * 1024;
+constexpr size_t kMaxPropSmem = 200 * 1024;  // flow and state of a tile's region (or a cluster block) at most
+constexpr size_t kMaxTileSmem = 216 * 1024;  // a tile launch's dynamic shared memory at most
 constexpr int kMaxCluster = 16;
-size_t prop_smem_bytes(int tw, int th, int n_iter);
+size_t prop_smem_bytes(int tw, int th, int n_iter);   // flow and state words of a tile's region: what limits a tile
+size_t prop_launch_smem(int tw, int th, int n_iter, bool listed);  // dynamic shared memory of a launch with that tile
+// The largest tiles prop_smem_bytes allows are shrunk to what a launch of the listed variant can take (results do not
+// depend on the tiles).
+void prop_fit_tile(int& tw, int& th);
+// Whether a pass of that many pixels (all problems of its launch), in tiles tw wide on CTAs of that many threads, takes
+// the listed variant of the dataflow form.
+bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow);
 
 // Cluster form of a propagation launch: the n CTAs of a cluster split a w x h problem into bx x by blocks
 // (bx * by = n), CTA r owning block (r % bx, r / bx) with columns [i*w/bx, (i+1)*w/bx) and rows
@@ -216,14 +225,14 @@ cudaError_t seed_load_kernel();        // loads k_seed onto the current device (
 cudaError_t noalloc_prepare(void** scratch);
 bool prop_threads_ok(int threads);
 // resident CTAs per SM of the tile form (dataflow: of its dataflow kernel)
-int prop_blocks_per_sm(size_t smem, int threads, bool spec, int cost, bool grid = false, bool dataflow = false);
+int prop_blocks_per_sm(size_t smem, int threads, int cost, bool dataflow, bool listed);
 // Tile form (L.cluster == 0): queue_dev[i] = (problem index, tile index); counter_dev must be zero when the launch
 // starts; `grid` CTAs.  Dataflow form (L.dataflow = T): the same queue, taken T times (iteration-major).  Cluster form: problem i is probs_dev[i], `grid` = number of problems x L.cluster CTAs;
 // queue_dev and counter_dev are unused.
 void launch_propagate(const PropProblem* probs_dev, const int2* queue_dev, int n_tiles, int* counter_dev, int grid,
                       const PropLaunch& L, cudaStream_t st);
 // Clusters of the cluster form that can be resident at once (0: this shape cannot be launched).
-int prop_cluster_capacity(int cluster, int threads, int cost, bool grid, size_t smem);
+int prop_cluster_capacity(int cluster, int threads, int cost, size_t smem);
 
 // ---------------------------------------------------------------------------------------------------------
 // consistency
@@ -268,7 +277,8 @@ struct CtxView {
     int* err_word;          // device error word of the bounded waits (null until ctx_err_word)
 };
 struct TileChoice {
-    int tw, th, k, threads, spec;
+    int tw, th, k, threads;
+    bool listed;   // the variant (prop_listed)
     int dataflow;  // 1: the dataflow form (k = iters: one launch per pass), 2: its affine variant; 0: tile form
 };
 

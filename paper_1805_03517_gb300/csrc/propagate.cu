@@ -14,7 +14,12 @@
 // value the remaining half-sweeps need: the region grows backwards from the tile by one pixel on the two
 // upstream sides of each later half-sweep.  Recomputed halo pixels use exactly the inputs of the CTA that owns
 // them, so every tile's output equals the global schedule bit for bit.
+//
+// The work of a tile has two variants.  The direct one gives every pixel of a half-sweep a thread, which scores the
+// pixel's candidates.  The listed one skips the candidates that are known not to be cheaper and gives threads only to
+// the pixels left (see there); dataflow launches of enough pixels to keep the GPU busy take it (prop_listed).
 #include <climits>
+#include <cstddef>
 
 #include "ff_internal.h"
 
@@ -35,7 +40,7 @@ cudaError_t bounds_take_propagate(int rec[3]) {
 }
 
 // Bounds codes of this file's checks.
-enum : int { kBoundsOwn = 1, kBoundsCand1, kBoundsCand2, kBoundsRandom, kBoundsSpec, kBoundsSmemOwn, kBoundsSmemN1,
+enum : int { kBoundsOwn = 1, kBoundsCand1, kBoundsCand2, kBoundsRandom, kBoundsSmemOwn, kBoundsSmemN1,
              kBoundsSmemN2, kBoundsTileRead, kBoundsTileSmem, kBoundsTileWrite, kBoundsParent, kBoundsHandoverDesc,
              kBoundsBlockRead, kBoundsBlockSmem, kBoundsBlockWrite, kBoundsRingN1, kBoundsRingN2 };
 
@@ -46,83 +51,89 @@ __device__ __forceinline__ bool in_level(int x, int y, int w, int h) {
     return (unsigned)x < (unsigned)w && (unsigned)y < (unsigned)h;
 }
 
-// One pixel descriptor (96 B = three 32-B sectors) with three 256-bit read-only loads, one sector per load.
-__device__ __forceinline__ void load_desc(const void* __restrict__ f, int idx, uint32_t (&d)[24]) {
-    const char* p = reinterpret_cast<const char*>(f) + (size_t)idx * kDescBytes;
-#pragma unroll
-    for (int k = 0; k < 3; k++)
-        asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=r"(d[8 * k]), "=r"(d[8 * k + 1]), "=r"(d[8 * k + 2]), "=r"(d[8 * k + 3]), "=r"(d[8 * k + 4]),
-              "=r"(d[8 * k + 5]), "=r"(d[8 * k + 6]), "=r"(d[8 * k + 7])
-            : "l"(p + 32 * k));
+// Eight 32-bit words (one 32-B sector of a descriptor) with one 256-bit read-only load.
+__device__ __forceinline__ void load_words8(const char* p, uint32_t (&d)[8]) {
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7])
+        : "l"(p));
 }
 
-// Exact SAD of the 48 coefficients, two per 32-bit word.  The feature maps store every coefficient in offset
-// binary (C ^ 0x8000, i.e. C + 32768 as uint16, which preserves order), so per half max - min is |a - b| in
+// The two matching costs (Sec. 3.1), as policies of the hand-over and propagation kernels: 32-B sectors per
+// descriptor, load of one sector, and the sector's share of the distance.  Every share is non-negative, so the sum
+// over the first sectors bounds the distance from below.
+//
+// SAD of the 48 WHT coefficients, one colour channel per sector.  The feature maps store every coefficient in
+// offset binary (C ^ 0x8000, i.e. C + 32768 as uint16, which preserves order), so per half max - min is |a - b| in
 // [0, 32640] and a plain 32-bit subtraction of the packed max/min never borrows across halves.  Two packed
-// differences add without carrying (2 * 32640 < 65536); __dp2a_lo then adds both 16-bit halves into the int32
-// sum.
-__device__ __forceinline__ int sad_words(const uint32_t (&a)[24], const uint32_t (&b)[24]) {
-    unsigned s = 0;
+// differences add without carrying (2 * 32640 < 65536); __dp2a_lo then adds both 16-bit halves into the int32 sum.
+// The 64 products of the 8x8 transform are orthogonal, so a channel's difference of two patches (each |difference|
+// <= 255) has a Euclidean norm of at most 64 * 255 and its 16 coefficients an absolute sum of at most 4 * 64 * 255:
+// a distance is at most 3 * 65280 = 195,840 < 2^18.
+struct CostSad {
+    static constexpr int kSectors = 3;
+    __device__ __forceinline__ static void load(const void* __restrict__ f, int idx, int k, uint32_t (&d)[8]) {
+        load_words8(reinterpret_cast<const char*>(f) + (size_t)idx * kDescBytes + 32 * k, d);
+    }
+    __device__ __forceinline__ static int dist(const uint32_t (&a)[8], const uint32_t (&b)[8], int s0) {
+        unsigned s = (unsigned)s0;
 #pragma unroll
-    for (int k = 0; k < 24; k += 2) {
-        uint32_t d0 = __vmaxu2(a[k], b[k]) - __vminu2(a[k], b[k]);
-        uint32_t d1 = __vmaxu2(a[k + 1], b[k + 1]) - __vminu2(a[k + 1], b[k + 1]);
-        s = __dp2a_lo(d0 + d1, 0x0101u, s);
-    }
-    return (int)s;
-}
-
-// The two matching costs (Sec. 3.1), as policies of the hand-over and propagation kernels: descriptor size in
-// 32-bit words, load of one pixel's descriptor, one-time preparation of the source pixel's descriptor, distance.
-struct CostSad {  // SAD of the 48 WHT coefficients (stored in offset binary)
-    static constexpr int kWords = 24;
-    __device__ __forceinline__ static void load(const void* __restrict__ f, int idx, uint32_t (&d)[kWords]) {
-        load_desc(f, idx, d);
-    }
-    __device__ __forceinline__ static void prep(uint32_t (&)[kWords]) {}
-    __device__ __forceinline__ static int dist(const uint32_t (&a)[kWords], const uint32_t (&b)[kWords]) {
-        return sad_words(a, b);
+        for (int k = 0; k < 8; k += 2) {
+            uint32_t d0 = __vmaxu2(a[k], b[k]) - __vminu2(a[k], b[k]);
+            uint32_t d1 = __vmaxu2(a[k + 1], b[k + 1]) - __vminu2(a[k + 1], b[k + 1]);
+            s = __dp2a_lo(d0 + d1, 0x0101u, s);
+        }
+        return (int)s;
     }
 };
 
-struct CostCensus {  // Hamming distance of the three 48-bit Census patterns (one 32-B sector per pixel)
-    static constexpr int kWords = 8;
-    __device__ __forceinline__ static void load(const void* __restrict__ f, int idx, uint32_t (&d)[kWords]) {
-        const char* p = reinterpret_cast<const char*>(f) + (size_t)idx * kCensusBytes;
-        asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7])
-            : "l"(p));
+// Hamming distance of the three 48-bit Census patterns (one sector per pixel; its words 6 and 7 are zero).
+struct CostCensus {
+    static constexpr int kSectors = 1;
+    __device__ __forceinline__ static void load(const void* __restrict__ f, int idx, int, uint32_t (&d)[8]) {
+        load_words8(reinterpret_cast<const char*>(f) + (size_t)idx * kCensusBytes, d);
     }
-    __device__ __forceinline__ static void prep(uint32_t (&)[kWords]) {}
-    __device__ __forceinline__ static int dist(const uint32_t (&a)[kWords], const uint32_t (&b)[kWords]) {
-        int s = 0;
+    __device__ __forceinline__ static int dist(const uint32_t (&a)[8], const uint32_t (&b)[8], int s) {
 #pragma unroll
-        for (int k = 0; k < 6; k++) s += __popc(a[k] ^ b[k]);  // words 6 and 7 are zero
+        for (int k = 0; k < 6; k++) s += __popc(a[k] ^ b[k]);
         return s;
     }
 };
 
-// A descriptor load that a debug-bounds build checks against the map's n descriptors (zeros if outside).
+// One sector of descriptor idx; a debug-bounds build checks the index against the map's n descriptors (zeros if
+// outside).
 template <class C>
-__device__ __forceinline__ void load_chk(const void* __restrict__ f, int idx, int n, int code, uint32_t (&d)[C::kWords]) {
+__device__ __forceinline__ void load_chk(const void* __restrict__ f, int idx, int n, int code, int k, uint32_t (&d)[8]) {
     if (idx_ok(g_bounds, code, idx, n)) {
-        C::load(f, idx, d);
+        C::load(f, idx, k, d);
     } else {
 #pragma unroll
-        for (int k = 0; k < C::kWords; k++) d[k] = 0;
+        for (int i = 0; i < 8; i++) d[i] = 0;
     }
+}
+
+// A whole descriptor.
+template <class C>
+__device__ __forceinline__ void load_all(const void* __restrict__ f, int idx, int n, int code,
+                                         uint32_t (&d)[C::kSectors][8]) {
+#pragma unroll
+    for (int k = 0; k < C::kSectors; k++) load_chk<C>(f, idx, n, code, k, d[k]);
+}
+template <class C>
+__device__ __forceinline__ int dist_all(const uint32_t (&a)[C::kSectors][8], const uint32_t (&b)[C::kSectors][8]) {
+    int s = 0;
+#pragma unroll
+    for (int k = 0; k < C::kSectors; k++) s = C::dist(a[k], b[k], s);
+    return s;
 }
 
 // Cost of the descriptor at (x, y) of fa against (tx, ty) of fb (both inside the w x h level).
 template <class C>
 __device__ __forceinline__ int cost_at(const void* __restrict__ fa, const void* __restrict__ fb, int w, int h, int x,
                                        int y, int tx, int ty) {
-    uint32_t a[C::kWords], b[C::kWords];
-    load_chk<C>(fa, feat_index(x, y, w), w * h, kBoundsHandoverDesc, a);
-    load_chk<C>(fb, feat_index(tx, ty, w), w * h, kBoundsHandoverDesc, b);
-    C::prep(a);
-    return C::dist(a, b);
+    uint32_t a[C::kSectors][8], b[C::kSectors][8];
+    load_all<C>(fa, feat_index(x, y, w), w * h, kBoundsHandoverDesc, a);
+    load_all<C>(fb, feat_index(tx, ty, w), w * h, kBoundsHandoverDesc, b);
+    return dist_all<C>(a, b);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -187,6 +198,24 @@ size_t prop_smem_bytes(int tw, int th, int n_iter) {
     return (size_t)(tw + 2 * H) * (th + 2 * H) * 8;
 }
 
+// The key of iteration t's random offsets, and of level pixel (X, Y) in it.
+__device__ __forceinline__ uint32_t iter_key(const PropProblem& P, int t) {
+    return mix32(P.seed ^ mix32((uint32_t)P.dir * 65536u + (uint32_t)P.level * 256u + (uint32_t)t));
+}
+__device__ __forceinline__ uint32_t pixel_key(uint32_t k1, int X, int Y) {
+    return mix32(k1 ^ ((uint32_t)Y * 65536u + (uint32_t)X));
+}
+
+// Where a tile task reads the state of its region and writes its interior, and which iterations it runs.
+struct TileIO {
+    const uint32_t* flow_in;
+    const int32_t* cost_in;
+    uint32_t* flow_out;
+    int32_t* cost_out;
+    int t0, n_iter;
+};
+
+// ---- direct variant
 
 // Geometry of the tile a CTA is working on (all coordinates are level coordinates).
 struct TileGeom {
@@ -211,31 +240,25 @@ __device__ __forceinline__ bool region_pixel(int i, int HW, int rx0, int ry0, in
     return x < rx1;
 }
 
-// The candidates of one pixel (x, y) of a grid in a half-sweep of direction d, one thread per pixel (the whole
-// descriptor per thread: 96 B WHT, 32 B Census): neighbour 1 (horizontal, flow f1, valid if v1), neighbour 2
-// (vertical, f2, v2) and, for d >= 1, the hashed random offset around the flow after them.  cur / c hold the
-// pixel's flow and cost and are updated; false if there was nothing to try (they are unchanged).  With SPEC the
-// random candidate of directions 1..3 is fetched together with the neighbour candidates, assuming the neighbours
-// will not change the pixel's flow; if one of them is taken, the random candidate is fetched again from the new
-// flow.  Either way the candidate evaluated is the one the schedule defines, so results are identical.
-// (Fetching it early only into a buffer no neighbour needs, without SPEC, measured 16 % slower on the 1242x375
-// pair.)
-// Per-launch constants of update_pixel, read from the problem once per half-sweep.
+// Per-launch constants of update_direct, read from the problem once per half-sweep.
 struct SweepConst {
     int g, lw, lh;  // grid stride and level size: grid pixel (x, y) is level pixel (g*x, g*y)
     int R;          // random-search radius
     uint32_t span;  // 2R + 1
 };
-template <bool GRID>
-__device__ __forceinline__ SweepConst sweep_const(const PropProblem& P) {
+__device__ __forceinline__ SweepConst sweep_const(const PropProblem& P, bool grid) {
     const int R = P.rs_radius;
-    return {GRID ? P.g : 1, GRID ? P.lw : P.w, GRID ? P.lh : P.h, R, 2u * R + 1u};
+    return {grid ? P.g : 1, grid ? P.lw : P.w, grid ? P.lh : P.h, R, 2u * R + 1u};
 }
 
-template <class C, bool SPEC, bool GRID>
-__device__ __forceinline__ bool update_pixel(const PropProblem& P, const SweepConst& K, int x, int y, int d,
-                                             uint32_t k1, bool v1, uint32_t f1, bool v2, uint32_t f2, uint32_t& cur,
-                                             int& c) {
+// The candidates of one pixel (x, y) of a grid in a half-sweep of direction d, one thread per pixel (the whole
+// descriptor per thread: 96 B WHT, 32 B Census): neighbour 1 (horizontal, flow f1, valid if v1), neighbour 2
+// (vertical, f2, v2) and, for d >= 1, the hashed random offset around the flow after them.  cur / c hold the
+// pixel's flow and cost and are updated; false if there was nothing to try (they are unchanged).
+template <class C>
+__device__ __forceinline__ bool update_direct(const PropProblem& P, const SweepConst& K, int x, int y, int d,
+                                              uint32_t k1, bool v1, uint32_t f1, bool v2, uint32_t f2, uint32_t& cur,
+                                              int& c) {
     // flows and targets are in level pixels
     const int g = K.g, lw = K.lw, lh = K.lh, R = K.R;
     const uint32_t span = K.span;
@@ -247,64 +270,46 @@ __device__ __forceinline__ bool update_pixel(const PropProblem& P, const SweepCo
     if (!(e1 || e2 || d >= 1)) return false;
     int ox = 0, oy = 0;
     if (d >= 1) {
-        const uint32_t k2 = mix32(k1 ^ ((uint32_t)Y * 65536u + (uint32_t)X));
+        const uint32_t k2 = pixel_key(k1, X, Y);
         ox = (int)(mix32(k2 ^ (uint32_t)(2 * d)) % span) - R;
         oy = (int)(mix32(k2 ^ (uint32_t)(2 * d + 1)) % span) - R;
     }
     const bool rnd = ox != 0 || oy != 0;
-    const uint32_t cur0 = cur;
-    // issue every independent load (own descriptor, neighbour candidates, speculative random) before compute
-    uint32_t a[C::kWords], b1[C::kWords], b2[C::kWords];
-    uint32_t b3[SPEC ? C::kWords : 1];
-    load_chk<C>(P.fa, feat_index(X, Y, lw), n_d, kBoundsOwn, a);
-    if (e1) load_chk<C>(P.fb, feat_index(X + flow_x(f1), Y + flow_y(f1), lw), n_d, kBoundsCand1, b1);
-    if (e2) load_chk<C>(P.fb, feat_index(X + flow_x(f2), Y + flow_y(f2), lw), n_d, kBoundsCand2, b2);
-    if constexpr (SPEC) {
-        const int sx = flow_x(cur) + ox, sy = flow_y(cur) + oy;
-        if (rnd && in_level(X + sx, Y + sy, lw, lh))
-            load_chk<C>(P.fb, feat_index(X + sx, Y + sy, lw), n_d, kBoundsSpec, b3);
-    }
-    C::prep(a);
+    // issue every independent load (own descriptor, neighbour candidates) before compute
+    uint32_t a[C::kSectors][8], b1[C::kSectors][8], b2[C::kSectors][8];
+    load_all<C>(P.fa, feat_index(X, Y, lw), n_d, kBoundsOwn, a);
+    if (e1) load_all<C>(P.fb, feat_index(X + flow_x(f1), Y + flow_y(f1), lw), n_d, kBoundsCand1, b1);
+    if (e2) load_all<C>(P.fb, feat_index(X + flow_x(f2), Y + flow_y(f2), lw), n_d, kBoundsCand2, b2);
     if (e1) {
-        int s1 = C::dist(a, b1);
+        int s1 = dist_all<C>(a, b1);
         if (s1 < c) { cur = f1; c = s1; }
     }
     if (e2) {
-        int s2 = C::dist(a, b2);
+        int s2 = dist_all<C>(a, b2);
         if (s2 < c) { cur = f2; c = s2; }
     }
     if (rnd) {
         const int fx = flow_x(cur) + ox, fy = flow_y(cur) + oy;
         if (in_level(X + fx, Y + fy, lw, lh)) {
-            int s3;
-            if constexpr (SPEC) {
-                if (cur == cur0) {
-                    s3 = C::dist(a, b3);  // same target as speculated (which was then in the level)
-                } else {
-                    load_chk<C>(P.fb, feat_index(X + fx, Y + fy, lw), n_d, kBoundsRandom, b1);
-                    s3 = C::dist(a, b1);
-                }
-            } else {
-                load_chk<C>(P.fb, feat_index(X + fx, Y + fy, lw), n_d, kBoundsRandom, b1);
-                s3 = C::dist(a, b1);
-            }
+            load_all<C>(P.fb, feat_index(X + fx, Y + fy, lw), n_d, kBoundsRandom, b1);
+            const int s3 = dist_all<C>(a, b1);
             if (s3 < c) { cur = pack_flow(fx, fy); c = s3; }
         }
     }
     return true;
 }
 
-// One half-sweep of a tile's region (tile form).
-template <class C, bool SPEC, bool GRID>
-__device__ __forceinline__ void halfsweep(const PropProblem& P, const TileGeom& G, uint32_t* sflow, int32_t* scost,
-                                          int j, int rem, uint32_t k1) {
-    const int w = P.w, h = P.h;  // the grid (the level itself unless GRID)
+// One half-sweep of a tile's region (direct variant).
+template <class C>
+__device__ __forceinline__ void halfsweep_direct(const PropProblem& P, const TileGeom& G, uint32_t* sflow,
+                                                 int32_t* scost, int j, int rem, uint32_t k1, bool grid) {
+    const int w = P.w, h = P.h;  // the grid (the level itself unless g > 1)
     const int d = j >> 1, colour = j & 1;
     int rx0, ry0, rx1, ry1;
     halfsweep_region(G, w, h, j, rem, rx0, ry0, rx1, ry1);
     const int HW = (rx1 - rx0 + 1) >> 1;
     const int total = HW * (ry1 - ry0);
-    const SweepConst K = sweep_const<GRID>(P);
+    const SweepConst K = sweep_const(P, grid);
     for (int i = threadIdx.x; i < total; i += blockDim.x) {
         int x, y;
         if (!region_pixel(i, HW, rx0, ry0, rx1, colour, x, y)) continue;
@@ -320,29 +325,19 @@ __device__ __forceinline__ void halfsweep(const PropProblem& P, const TileGeom& 
         const uint32_t f1 = v1 && idx_ok(g_bounds, kBoundsSmemN1, sidx + (n1x - x), n_s) ? sflow[sidx + (n1x - x)] : 0u;
         const uint32_t f2 =
             v2 && idx_ok(g_bounds, kBoundsSmemN2, sidx + (n2y - y) * G.RW, n_s) ? sflow[sidx + (n2y - y) * G.RW] : 0u;
-        if (!update_pixel<C, SPEC, GRID>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) continue;
+        if (!update_direct<C>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) continue;
         sflow[sidx] = cur;
         scost[sidx] = c;
     }
 }
 
-// Where a tile task reads the state of its region and writes its interior, and which iterations it runs.
-struct TileIO {
-    const uint32_t* flow_in;
-    const int32_t* cost_in;
-    uint32_t* flow_out;
-    int32_t* cost_out;
-    int t0, n_iter;
-};
-
 // One tile of one problem: load the tile and its halo, run n_iter iterations in shared memory, write the tile.
-// The buffers and iterations are the problem's (tile form) or, with DF, those of `io`, a dataflow task whose
-// state was written by other CTAs of the running launch and is therefore read from L2.
-template <class C, bool SPEC, bool GRID, bool DF = false>
-__device__ __forceinline__ void propagate_tile(const PropProblem& P, int tile, const PropLaunch& L, uint32_t* smem,
-                                               const TileIO* io = nullptr) {
+// With DF, a dataflow task, the state was written by other CTAs of the running launch and is therefore read from L2.
+template <class C, bool DF>
+__device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int tile, const PropLaunch& L,
+                                                      uint32_t* smem, const TileIO& io) {
     const int w = P.w, h = P.h;
-    const int n_iter = DF ? io->n_iter : P.n_iter;
+    const int n_iter = io.n_iter;
     TileGeom G;
     G.x0 = (tile % P.tiles_x) * L.tw;
     G.y0 = (tile / P.tiles_x) * L.th;
@@ -362,21 +357,16 @@ __device__ __forceinline__ void propagate_tile(const PropProblem& P, int tile, c
         // flow and cost of the region (2 words per pixel) must fit the launch's dynamic shared memory
         const bool ok = idx_ok(g_bounds, kBoundsTileRead, (long long)g, (long long)w * h) &&
                         (!FF_DEBUG_BOUNDS || idx_ok(g_bounds, kBoundsTileSmem, 2 * G.RW * G.RH - 1, dyn_smem_bytes() / 4));
-        if constexpr (DF) {
-            sflow[i] = ok ? __ldcg(io->flow_in + g) : 0u;
-            scost[i] = ok ? __ldcg(io->cost_in + g) : 0;
-        } else {
-            sflow[i] = ok ? P.flow_in[g] : 0u;
-            scost[i] = ok ? P.cost_in[g] : 0;
-        }
+        sflow[i] = !ok ? 0u : DF ? __ldcg(io.flow_in + g) : io.flow_in[g];
+        scost[i] = !ok ? 0 : DF ? __ldcg(io.cost_in + g) : io.cost_in[g];
     }
     __syncthreads();
     for (int it = 0; it < n_iter; it++) {
-        const int t = (DF ? io->t0 : P.t0) + it;
+        const int t = io.t0 + it;
         const int rem = kHaloPerIter * (n_iter - 1 - it);
-        const uint32_t k1 = mix32(P.seed ^ mix32((uint32_t)P.dir * 65536u + (uint32_t)P.level * 256u + (uint32_t)t));
+        const uint32_t k1 = iter_key(P, t);
         for (int j = 0; j < 8; j++) {
-            halfsweep<C, SPEC, GRID>(P, G, sflow, scost, j, rem, k1);
+            halfsweep_direct<C>(P, G, sflow, scost, j, rem, k1, L.grid != 0);
             __syncthreads();
         }
     }
@@ -388,21 +378,495 @@ __device__ __forceinline__ void propagate_tile(const PropProblem& P, int tile, c
         if (!idx_ok(g_bounds, kBoundsTileWrite, (long long)g, (long long)w * h) ||
             !idx_ok(g_bounds, kBoundsTileSmem, sidx, G.RW * G.RH))
             continue;
-        (DF ? io->flow_out : P.flow_out)[g] = sflow[sidx];
-        (DF ? io->cost_out : P.cost_out)[g] = scost[sidx];
+        io.flow_out[g] = sflow[sidx];
+        io.cost_out[g] = scost[sidx];
     }
+}
+
+// ---- listed variant (dataflow form)
+//
+// What bounds the direct variant at level 0 of the 1242x375 pair is gathers and instructions alike: 28.9 M sectors
+// and 59 M instructions per iteration, most of them for candidates that are known not to be cheaper, at 44 % of the
+// issue slots.  This variant loads 13 M sectors per iteration and runs 32 instead of 16 warps per SM: level 0 in 567
+// instead of 663 us (all six iterations), of the 1920x1080 pair in 1816 instead of 2760.
+
+// What a pixel still has to try, one byte per pixel in shared memory.  Costs only fall and
+// a candidate's cost is fixed, so a candidate that was not cheaper than a pixel's flow never becomes so: a
+// neighbour's flow needs a trial only if it changed since the pixel last tried that neighbour, and a random candidate
+// that the screening found not cheaper needs none while the pixel keeps its flow.  On the 1242x375 pair this leaves,
+// per pixel and iteration of level 0, 2.0, 1.3, 0.6, 0.4, 0.3 and 0.25 neighbour trials in iterations 0..5 instead of
+// 2.3 to 3.0; results are the same bit for bit.
+//   bits 0..3  the left, right, upper, lower neighbour's flow has changed since its last trial
+//   bits 4..6  the random candidate of direction 1, 2, 3 has to be scored
+constexpr uint32_t kTodoAll = 0x7f7f7f7fu;
+__device__ __forceinline__ uint32_t todo_bits(int d) {  // those of direction d
+    return (1u << (d & 1)) | (4u << (d >> 1)) | (d ? 8u << d : 0u);
+}
+
+// The state word between the tasks of a pass (in the cost buffers):
+//   bits 31..14  cost of the flow (at most 195,840, see CostSad; Census 144)
+//   bits 13..11  the random candidates of the next iteration that have to be scored (screen)
+//   bits 3..0    1 + the half-sweep of the iteration that last changed the flow, 0: none did
+// In shared memory the flags are in the todo bytes.
+constexpr int kCostShift = 14, kFlagShift = 11;
+constexpr uint32_t kStampMask = 15u, kCostMax = (1u << (32 - kCostShift)) - 1;
+__device__ __forceinline__ uint32_t pack_state(int cost) { return min((uint32_t)cost, kCostMax) << kCostShift; }
+// Whom the change of a pixel's flow in half-sweep stamp - 1 still concerns when the next iteration starts: bit 0 the
+// pixel right of it (whose left neighbour it is), 1 left, 2 below, 3 above.  A pixel of colour k last tried its left
+// neighbour in half-sweep 4 + k, its right and lower ones in 6 + k, its upper one in 2 + k; one nibble per stamp.
+constexpr uint32_t still_concerned() {
+    uint32_t m = 0;
+    for (int s = 1; s <= 8; s++) {
+        const int j = s - 1, k = 1 - (j & 1);  // the neighbours have the other colour
+        const uint32_t n = (j > 4 + k ? 1u : 0u) | (j > 6 + k ? 2u : 0u) | (j > 2 + k ? 4u : 0u) | (j > 6 + k ? 8u : 0u);
+        m |= n << (4 * (s - 1));
+    }
+    return m;
+}
+
+// Constants of a problem, in shared memory.
+struct alignas(16) Sweep {
+    const void* fa;
+    const void* fb;
+    int g, lw, lh, half;  // grid stride and level size: grid pixel (x, y) is level pixel (g*x, g*y); (lw + 1) / 2
+    uint32_t span, inv;   // 2R + 1 (R: random-search radius) and floor(2^32 / span)
+    int R, pad;
+    __device__ __forceinline__ void set(const PropProblem& P, bool grid) {
+        fa = P.fa;
+        fb = P.fb;
+        g = grid ? P.g : 1;
+        lw = grid ? P.lw : P.w;
+        lh = grid ? P.lh : P.h;
+        half = (lw + 1) >> 1;
+        R = P.rs_radius;
+        span = 2u * P.rs_radius + 1u;
+        inv = 0xffffffffu / span;  // (2^32 has the same quotient, except for span 1, where every offset is 0 anyway)
+    }
+};
+
+// Reads of CTA-wide constants in shared memory by address.  Every pixel takes a fresh copy of the address the compiler
+// cannot see through, so the constants are read where they are used (four at a time, a broadcast) and hold no
+// registers across the pixels.
+__device__ __forceinline__ uint32_t fresh(uint32_t a) {
+    asm volatile("" : "+r"(a));
+    return a;
+}
+__device__ __forceinline__ int4 lds_int4(uint32_t a) {
+    int4 v;
+    asm("ld.shared.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+struct SweepRef {
+    uint32_t a;  // address of a Sweep
+    __device__ __forceinline__ const void* ptr(uint32_t offset) const {
+        uint64_t v;
+        asm("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a + offset));
+        return reinterpret_cast<const void*>(v);
+    }
+    __device__ __forceinline__ const void* fa() const { return ptr(offsetof(Sweep, fa)); }
+    __device__ __forceinline__ const void* fb() const { return ptr(offsetof(Sweep, fb)); }
+    __device__ __forceinline__ int4 level() const { return lds_int4(a + (uint32_t)offsetof(Sweep, g)); }  // g, lw, lh, half
+    __device__ __forceinline__ int g() const { return level().x; }
+    // Descriptor of level pixel (X, Y) in the colour-split rows (feat_index).
+    __device__ __forceinline__ int index(int X, int Y) const {
+        const int4 L = level();
+        return Y * L.y + (X >> 1) + ((X & 1) ? L.w : 0);
+    }
+    __device__ __forceinline__ bool inside(int X, int Y) const {
+        const int4 L = level();
+        return in_level(X, Y, L.y, L.z);
+    }
+    __device__ __forceinline__ int n_desc() const {  // of the level (debug-bounds checks)
+        return FF_DEBUG_BOUNDS ? level().y * level().z : 0;
+    }
+    // hash % span - R; the quotient is at most one too small
+    __device__ __forceinline__ static int offset(uint32_t hash, const int4& r) {
+        const uint32_t span = (uint32_t)r.x, m = hash - __umulhi(hash, (uint32_t)r.y) * span;
+        return (int)(m >= span ? m - span : m) - r.z;
+    }
+    // The random offset of direction d for the pixel key k2.
+    __device__ __forceinline__ void random_offset(uint32_t k2, int d, int& ox, int& oy) const {
+        const int4 r = lds_int4(a + (uint32_t)offsetof(Sweep, span));  // span, inv, R
+        ox = offset(mix32(k2 ^ (uint32_t)(2 * d)), r);
+        oy = offset(mix32(k2 ^ (uint32_t)(2 * d + 1)), r);
+    }
+};
+
+// The candidates of one pixel (x, y) of a grid in a half-sweep of direction d, one thread per pixel: neighbour 1
+// (horizontal, flow f1, to be tried if t1), neighbour 2 (vertical, f2, t2) and, for d >= 1, the hashed random
+// offset around the flow after them.  The random candidate is scored if `rnd`, or if a neighbour was taken (else it
+// is known not to be cheaper).  cur / c hold the pixel's flow and cost and are updated.
+// (The descriptors are cleared where a load may be left out: a register that a predicated load may leave unwritten
+// stays reserved through every enclosing loop, which cost 30 to 50 registers a thread and half of the warps.)
+template <class C>
+__device__ __forceinline__ void update_pixel(const SweepRef K, int x, int y, int d, uint32_t k1, bool t1, uint32_t f1,
+                                             bool t2, uint32_t f2, bool rnd, uint32_t& cur, int& c) {
+    const int g = K.g(), X = g * x, Y = g * y;  // level coordinates, in which flows and targets are
+    const int n_d = K.n_desc();
+    // a candidate equal to the current flow (or to an already tried one) cannot be strictly cheaper
+    const bool e1 = t1 && f1 != cur && K.inside(X + flow_x(f1), Y + flow_y(f1));
+    const bool e2 = t2 && f2 != cur && !(t1 && f2 == f1) && K.inside(X + flow_x(f2), Y + flow_y(f2));
+    const int own = K.index(X, Y);
+    const uint32_t cur0 = cur;
+    uint32_t a[C::kSectors][8] = {};  // the own descriptor, kept if the neighbours are scored
+    const bool nb = e1 || e2;
+    if (nb) {
+        const int i1 = e1 ? K.index(X + flow_x(f1), Y + flow_y(f1)) : 0;
+        const int i2 = e2 ? K.index(X + flow_x(f2), Y + flow_y(f2)) : 0;
+        int s1 = 0, s2 = 0;
+#pragma unroll
+        for (int k = 0; k < C::kSectors; k++) {
+            uint32_t b1[8] = {}, b2[8] = {};
+            load_chk<C>(K.fa(), own, n_d, kBoundsOwn, k, a[k]);
+            if (e1) load_chk<C>(K.fb(), i1, n_d, kBoundsCand1, k, b1);
+            if (e2) load_chk<C>(K.fb(), i2, n_d, kBoundsCand2, k, b2);
+            if (e1) s1 = C::dist(a[k], b1, s1);
+            if (e2) s2 = C::dist(a[k], b2, s2);
+        }
+        if (e1 && s1 < c) { cur = f1; c = s1; }
+        if (e2 && s2 < c) { cur = f2; c = s2; }
+    }
+    if (d >= 1 && (rnd || cur != cur0)) {
+        int ox, oy;
+        K.random_offset(pixel_key(k1, X, Y), d, ox, oy);
+        const int fx = flow_x(cur) + ox, fy = flow_y(cur) + oy;
+        if ((ox != 0 || oy != 0) && K.inside(X + fx, Y + fy)) {
+            const int i3 = K.index(X + fx, Y + fy);
+            int s3 = 0;
+#pragma unroll
+            for (int k = 0; k < C::kSectors; k++)
+                if (s3 < c) {  // (a partial distance that reaches the cost settles it)
+                    uint32_t b[8];
+                    if (!nb) load_chk<C>(K.fa(), own, n_d, kBoundsOwn, k, a[k]);
+                    load_chk<C>(K.fb(), i3, n_d, kBoundsRandom, k, b);
+                    s3 = C::dist(a[k], b, s3);
+                }
+            if (s3 < c) { cur = pack_flow(fx, fy); c = s3; }
+        }
+    }
+}
+
+// Shared memory of a CTA of the tile and dataflow forms: the head, then for the region (tile + halo, clipped to the
+// grid) flow words and state words, row by row, todo bytes and the list.  A row has 2^(slots + 1) pixels (the region's
+// width rounded up to a power of two, so that places are shifts and masks).  The todo bytes and the list index the
+// pixels of a colour: slot b = (ry + 1) << slots | rx >> 1 for region pixel (rx, ry).  The todo bytes have a row of
+// padding above and below the region, so that a pixel's neighbours always have a byte (a mark that runs over the side
+// of a row falls on another pixel of the region and only costs it a needless trial).  The layout is one launch's.
+struct alignas(16) TileShared {
+    Sweep K;
+    int lx0, ly0, w, h;    // first pixel of the region, size of the grid
+    int x0, y0, x1, y1;    // tile interior
+    int RW, RH;            // region
+    int4 rect[8];          // region of half-sweep j relative to the loaded region: x0, y0, x1, y1
+    int n_list[8];         // its list entries
+    TileIO io;
+};
+constexpr int kHeadWords = 96;
+static_assert(sizeof(TileShared) <= 4 * kHeadWords, "head of the shared memory");
+constexpr int kMaxSlots = 1 << 13;  // slots a list entry can index
+
+struct TileLayout {
+    int slots, rows;  // log2 of the slots of a row; rows of the region
+    __host__ __device__ int n_pixels() const { return (2 * rows) << slots; }
+    __host__ __device__ int n_slots() const { return (rows + 2) << slots; }  // with the padding
+    __host__ __device__ int o_state() const { return kHeadWords + n_pixels(); }
+    __host__ __device__ int o_todo() const { return o_state() + n_pixels(); }
+    __host__ __device__ int todo_words() const { return n_slots() >> 2; }  // per colour
+    __host__ __device__ int o_list() const { return o_todo() + 2 * todo_words(); }
+    __host__ size_t bytes() const { return 4 * (size_t)o_list() + 2 * (size_t)n_slots(); }
+};
+TileLayout tile_layout(int tw, int th) {
+    TileLayout T{2, th + 2 * kHaloPerIter};
+    while ((2 << T.slots) < tw + 2 * kHaloPerIter) T.slots++;
+    return T;
+}
+size_t prop_launch_smem(int tw, int th, int n_iter, bool listed) {
+    return listed ? tile_layout(tw, th).bytes() : prop_smem_bytes(tw, th, n_iter);
+}
+void prop_fit_tile(int& tw, int& th) {
+    for (;;) {
+        const TileLayout T = tile_layout(tw, th);
+        if (T.bytes() <= kMaxTileSmem && T.n_slots() <= kMaxSlots) return;
+        int& longer = th >= tw ? th : tw;
+        longer -= (longer + 7) / 8;
+    }
+}
+
+// The line between the variants, from both timed in their best tiles (all iterations of a pass, WHT-SAD, T = 6, us,
+// direct / listed): 167 k pixels 160 / 199, 232 k 235 / 250, 259 k 248 / 248, 346 k 297 / 293, 614 k 360 / 299, 932 k
+// 663 / 567, 1.04 M 708 / 551, 4.1 M 2760 / 1816, 5.6 M 3794 / 2800; Census 232 k 147 / 156, 614 k 266 / 217, 4.1 M 1649 /
+// 1050.  Below it a half-sweep's chain of dependent loads bounds a pass, not the amount of work, and the direct
+// variant's chain is the shorter one.  What does not suit the listed variant keeps the direct one: the tile form (one
+// 640x480 direction 795 us listed, 639 direct: a launch per iteration leaves the screening's tail exposed), 128 threads
+// (level 0 of the 1242x375 pair in 48x24 tiles: 900 us listed, 663 direct), and regions that leave over a quarter of
+// their power-of-two rows empty (64x32 tiles, 72 wide: 688, 669 direct).
+constexpr int64_t kListedPixels = 300000;
+bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow) {
+    const int RW = tw + 2 * kHaloPerIter;
+    int pitch = 8;
+    while (pitch < RW) pitch *= 2;
+    return dataflow && pass_pixels >= kListedPixels && threads >= 256 && 4 * RW >= 3 * pitch;
+}
+
+extern __shared__ __align__(16) uint32_t g_smem[];
+__device__ __forceinline__ TileShared& tile_shared() { return *reinterpret_cast<TileShared*>(g_smem); }
+__device__ __forceinline__ SweepRef tile_sweep() { return {fresh(smem_u32(g_smem)) + (uint32_t)offsetof(TileShared, K)}; }
+__device__ __forceinline__ int4 tile_origin() { return lds_int4(fresh(smem_u32(g_smem)) + (uint32_t)offsetof(TileShared, lx0)); }
+
+// The flow of the pixel of slot b changed: the neighbours (of the other colour, whose todo bytes these are) that look
+// at it and are in `who` (bit 0 the pixel to the right, 1 left, 2 below, 3 above) have it to try.  Of the pixels left
+// and right of it, one has the same slot.
+__device__ __forceinline__ void mark_neighbours(uint32_t* todo, int b, int slots, int rx, uint32_t who) {
+    const bool odd = rx & 1;
+    const int sh = 8 * (b & 3);
+    uint32_t* at = todo + (b >> 2);
+    if (who & 4u) atomicOr(at + (1 << slots >> 2), 4u << sh);
+    if (who & 8u) atomicOr(at - (1 << slots >> 2), 8u << sh);
+    if (who & (odd ? 2u : 1u)) atomicOr(at, (odd ? 2u : 1u) << sh);
+    const int side = odd ? b + 1 : b - 1;
+    if (who & (odd ? 1u : 2u)) atomicOr(todo + (side >> 2), (odd ? 1u : 2u) << (8 * (side & 3)));
+}
+
+// Screening of the random candidates of the next iteration, at the end of an iteration (k1: the next one's key): for
+// every pixel of the tile, the candidates of directions 1..3 around its present flow are scored side by
+// side, sector by sector, each until its partial distance reaches the pixel's cost.  A candidate that reaches it is
+// not cheaper, and stays so while the pixel keeps its flow; the others (a few per cent) are flagged in the state word
+// and scored again in their half-sweep, as are those of pixels whose flow has changed by then.  So the own descriptor is loaded once per iteration instead of once per
+// direction, candidates of matched pixels are mostly dropped after one of their three sectors, three gathers are in
+// flight per thread, the half-sweeps are left with few pixels, and a tile screens its own pixels only: the flags of
+// its halo come with the state its neighbours wrote.
+template <class C, int THREADS>
+__device__ __forceinline__ void screen(const TileLayout T, int colour, const int4 r, uint32_t k1) {
+    const int tid = (int)fresh(threadIdx.x);
+    const int HWr = (r.z - r.x + 1) >> 1, total = HWr * (r.w - r.y);
+    const uint32_t inv = 0xffffffffu / (uint32_t)HWr + 1u;  // ceil(2^32 / HWr): i / HWr = umulhi(i, inv) for i < 2^15
+#pragma unroll 1
+    for (int i = tid; i < total; i += THREADS) {
+        const int4 O = tile_origin();
+        const SweepRef K = tile_sweep();
+        const int row = HWr > 1 ? (int)__umulhi((uint32_t)i, inv) : i;
+        const int ry = r.y + row;
+        const int rx = r.x + 2 * (i - row * HWr) + ((O.x + O.y + r.x + ry + colour) & 1);
+        if (rx >= r.z) continue;
+        const int sidx = (ry << (T.slots + 1)) + rx;
+        if (!idx_ok(g_bounds, kBoundsSmemOwn, sidx, T.n_pixels())) continue;
+        const uint32_t cur = g_smem[kHeadWords + sidx];
+        const int c = (int)(g_smem[T.o_state() + sidx] >> kCostShift);
+        const int g = K.g(), X = g * (O.x + rx), Y = g * (O.y + ry), n_d = K.n_desc();
+        uint32_t live = 0;
+        int idx[3], s[3];
+        {
+            const int cx = X + flow_x(cur), cy = Y + flow_y(cur);
+            const uint32_t k2 = pixel_key(k1, X, Y);
+#pragma unroll
+            for (int q = 0; q < 3; q++) {
+                int ox, oy;
+                K.random_offset(k2, q + 1, ox, oy);
+                if ((ox != 0 || oy != 0) && K.inside(cx + ox, cy + oy)) live |= 1u << q;
+                idx[q] = K.index(cx + ox, cy + oy);
+                s[q] = 0;
+            }
+        }
+        const int own = K.index(X, Y);
+#pragma unroll
+        for (int k = 0; k < C::kSectors; k++) {
+            if (!live) break;
+            uint32_t a[8], b[3][8] = {};
+            load_chk<C>(K.fa(), own, n_d, kBoundsOwn, k, a);
+#pragma unroll
+            for (int q = 0; q < 3; q++)
+                if (live >> q & 1u) load_chk<C>(K.fb(), idx[q], n_d, kBoundsRandom, k, b[q]);
+#pragma unroll
+            for (int q = 0; q < 3; q++)
+                if (live >> q & 1u) {
+                    s[q] = C::dist(a, b[q], s[q]);
+                    if (s[q] >= c) live &= ~(1u << q);
+                }
+        }
+        if (live) g_smem[T.o_state() + sidx] |= live << kFlagShift;
+    }
+}
+
+// One half-sweep of a tile's region.  The CTA collects the pixels of the region's rows whose
+// todo bytes hold something to try in this direction in a list (four pixels per thread and read, placed by ballots and
+// one counter), and updates them from the list, one per thread: a half-sweep with few such pixels costs few gathers
+// and few instructions.  A list entry is the slot and three bits, what to try: neighbour 1, neighbour 2, random.
+template <class C, int THREADS>
+__device__ __forceinline__ void halfsweep(const TileLayout T, int j, uint32_t k1) {
+    const int tid = (int)fresh(threadIdx.x);
+    const int d = j >> 1, colour = j & 1;
+    uint32_t* const mine = g_smem + T.o_todo() + colour * T.todo_words();
+    uint16_t* const list = reinterpret_cast<uint16_t*>(g_smem + T.o_list());
+    {
+        const int4 r = tile_shared().rect[j];
+        const uint32_t bits = todo_bits(d) * 0x01010101u;
+        const int lane = tid & 31, w1 = (r.w + 1) << T.slots >> 2;
+#pragma unroll 1
+        for (int base = ((r.y + 1) << T.slots >> 2) + (tid & ~31); base < w1; base += THREADS) {
+            const int i = base + lane;
+            uint32_t v = 0;
+            if (i < w1) {
+                v = mine[i];
+                if (v & bits) mine[i] = v & ~bits;  // (a neighbour tried now needs no trial until it changes again)
+                v &= bits;
+            }
+            if (!__any_sync(0xffffffffu, v != 0)) continue;
+            uint32_t nz = (v + kTodoAll) & 0x80808080u;  // bit 7 of every byte with something to try
+            const unsigned cnt = __popc(nz), below = (1u << lane) - 1u;
+            const unsigned c0 = __ballot_sync(0xffffffffu, cnt & 1u), c1 = __ballot_sync(0xffffffffu, cnt & 2u),
+                           c2 = __ballot_sync(0xffffffffu, cnt & 4u);
+            int pos = 0;
+            if (lane == 0) pos = atomicAdd(&tile_shared().n_list[j], __popc(c0) + 2 * __popc(c1) + 4 * __popc(c2));
+            pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(c0 & below) + 2 * __popc(c1 & below) + 4 * __popc(c2 & below);
+#pragma unroll 1
+            while (nz) {
+                const int s = __ffs((int)nz) - 8;  // first bit of the byte
+                const uint32_t t = v >> s;
+                list[pos++] = (uint16_t)((uint32_t)(4 * i + (s >> 3)) | (t & 3u ? 0x2000u : 0u) | (t & 12u ? 0x4000u : 0u) |
+                                         (t & 0x70u ? 0x8000u : 0u));
+                nz &= nz - 1;
+            }
+        }
+    }
+    __syncthreads();
+    const int n = tile_shared().n_list[j];
+    if (n == 0) return;  // (uniform)
+#pragma unroll 1
+    for (int i = tid; i < n; i += THREADS) {
+        const uint32_t e = list[i];
+        const int4 O = tile_origin();
+        const int b = (int)(e & 0x1fffu), ry = (b >> T.slots) - 1;
+        const int rx = 2 * (b & ((1 << T.slots) - 1)) + ((O.x + O.y + ry + colour) & 1);
+        const int sidx = (ry << (T.slots + 1)) + rx;
+        const int4 r = lds_int4(fresh(smem_u32(&tile_shared().rect[j])));
+        if (rx < r.x || rx >= r.z || !idx_ok(g_bounds, kBoundsSmemOwn, sidx, T.n_pixels())) continue;
+        const int x = O.x + rx, y = O.y + ry;
+        uint32_t cur = g_smem[kHeadWords + sidx];
+        const uint32_t cur0 = cur;
+        int c = (int)(g_smem[T.o_state() + sidx] >> kCostShift);
+        const int n1 = sidx + ((d & 1) ? 1 : -1), n2 = sidx + ((d & 2) ? 2 << T.slots : -(2 << T.slots));
+        const bool t1 = (e & 0x2000u) && (unsigned)(x + ((d & 1) ? 1 : -1)) < (unsigned)O.z &&
+                        idx_ok(g_bounds, kBoundsSmemN1, n1, T.n_pixels());
+        const bool t2 = (e & 0x4000u) && (unsigned)(y + ((d & 2) ? 1 : -1)) < (unsigned)O.w &&
+                        idx_ok(g_bounds, kBoundsSmemN2, n2, T.n_pixels());
+        const uint32_t f1 = t1 ? g_smem[kHeadWords + n1] : 0u, f2 = t2 ? g_smem[kHeadWords + n2] : 0u;
+        update_pixel<C>(tile_sweep(), x, y, d, k1, t1, f1, t2, f2, (e & 0x8000u) != 0, cur, c);
+        if (cur != cur0) {
+            g_smem[kHeadWords + sidx] = cur;
+            g_smem[T.o_state() + sidx] = (uint32_t)c << kCostShift | (uint32_t)(j + 1);
+            mark_neighbours(g_smem + T.o_todo() + (colour ^ 1) * T.todo_words(), b, T.slots, rx, 15u);
+            if (d < 3) atomicOr(mine + (b >> 2), ((0x70u << d) & 0x70u) << (8 * (b & 3)));  // random candidates to come
+        }
+    }
+    __syncthreads();
+}
+
+// Regions of the half-sweeps, without list entries yet (threads 0..7).
+__device__ __forceinline__ void set_regions() {
+    const int j = threadIdx.x;
+    TileShared& S = tile_shared();
+    if (j < 8) {
+        S.rect[j] = make_int4(max(S.x0 - c_grow[j][0], 0) - S.lx0, max(S.y0 - c_grow[j][1], 0) - S.ly0,
+                              min(S.x1 + c_grow[j][2], S.w) - S.lx0, min(S.y1 + c_grow[j][3], S.h) - S.ly0);
+        S.n_list[j] = 0;
+    }
+}
+
+// One tile of one problem: load the tile and its halo, run iteration io.t0 in shared memory, write the tile.  The state
+// was written by other CTAs of the running launch and is therefore read from L2.  Between the tasks of a pass the cost buffers hold state words; a pass starts from plain costs and its last
+// iteration leaves plain costs.  The head of the shared memory is set (tile_setup).
+template <class C, int THREADS>
+__device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, const TileLayout T) {
+    TileShared& S = tile_shared();
+    {
+        uint32_t* todo = g_smem + T.o_todo();
+        const int RW = S.RW, n_s = RW * S.RH, n_todo = 2 * T.todo_words();
+        const bool first = S.io.t0 == 0;  // of the pass: everything is still to be tried
+#pragma unroll 1
+        for (int i = threadIdx.x; i < n_todo; i += THREADS)  // (nothing for the slots past the region's width)
+            todo[i] = first && 8 * (i & ((1 << T.slots >> 2) - 1)) < RW ? kTodoAll : 0u;
+        set_regions();
+        if (!first) __syncthreads();
+        const uint32_t inv = 0xffffffffu / (uint32_t)RW + 1u;
+#pragma unroll 1
+        for (int i = threadIdx.x; i < n_s; i += THREADS) {
+            const int r = RW > 1 ? (int)__umulhi((uint32_t)i, inv) : i, c = i - r * RW;
+            const size_t g = (size_t)(S.ly0 + r) * S.w + S.lx0 + c;
+            // the region must fit the launch's dynamic shared memory
+            const bool ok = idx_ok(g_bounds, kBoundsTileRead, (long long)g, (long long)S.w * S.h) &&
+                            (!FF_DEBUG_BOUNDS || (idx_ok(g_bounds, kBoundsTileSmem, RW - 1, 2 << T.slots) &&
+                                                  idx_ok(g_bounds, kBoundsTileSmem, S.RH - 1, T.rows) &&
+                                                  idx_ok(g_bounds, kBoundsTileSmem, 4 * T.o_list() + 2 * T.n_slots() - 1,
+                                                         dyn_smem_bytes())));
+            uint32_t f = 0, st = 0;
+            if (ok) {
+                f = __ldcg(S.io.flow_in + g);
+                st = (uint32_t)__ldcg(S.io.cost_in + g);
+            }
+            const int sidx = (r << (T.slots + 1)) + c;
+            g_smem[kHeadWords + sidx] = f;
+            g_smem[T.o_state() + sidx] = first ? pack_state((int)st) : st >> kCostShift << kCostShift;
+            if (!first && (st & ((1u << kCostShift) - 1))) {
+                const uint32_t live = st >> kFlagShift & 7u, stamp = st & kStampMask;
+                const uint32_t who = stamp ? still_concerned() >> (4 * (stamp - 1)) & 15u : 0u;
+                const int colour = (S.lx0 + c + S.ly0 + r) & 1, b = ((r + 1) << T.slots) + (c >> 1);
+                if (live) atomicOr(todo + colour * T.todo_words() + (b >> 2), live << (8 * (b & 3) + 4));
+                if (who) mark_neighbours(todo + (colour ^ 1) * T.todo_words(), b, T.slots, c, who);
+            }
+        }
+        __syncthreads();
+    }
+    const int t = S.io.t0;
+    const bool plain = t + 1 == P.T;
+    const uint32_t k1 = iter_key(P, t);
+#pragma unroll 1
+    for (int j = 0; j < 8; j++) halfsweep<C, THREADS>(T, j, k1);
+    if (!plain) {
+        const uint32_t kn = iter_key(P, t + 1);
+#pragma unroll 1
+        for (int colour = 0; colour < 2; colour++) screen<C, THREADS>(T, colour, S.rect[7], kn);  // the tile
+    }
+    __syncthreads();
+    const int TW = S.x1 - S.x0, n_out = TW * (S.y1 - S.y0);
+    const uint32_t inv = 0xffffffffu / (uint32_t)TW + 1u;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n_out; i += THREADS) {
+        const int r = TW > 1 ? (int)__umulhi((uint32_t)i, inv) : i, c = i - r * TW;
+        const int sidx = ((S.y0 + r - S.ly0) << (T.slots + 1)) + (S.x0 + c - S.lx0);
+        const size_t g = (size_t)(S.y0 + r) * S.w + S.x0 + c;
+        if (!idx_ok(g_bounds, kBoundsTileWrite, (long long)g, (long long)S.w * S.h) ||
+            !idx_ok(g_bounds, kBoundsTileSmem, sidx, T.n_pixels()))
+            continue;
+        S.io.flow_out[g] = g_smem[kHeadWords + sidx];
+        const uint32_t st = g_smem[T.o_state() + sidx];
+        S.io.cost_out[g] = (int32_t)(plain ? st >> kCostShift : st);
+    }
+}
+
+// Problem and geometry of the CTA's next tile, by one thread.
+__device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const PropLaunch& L) {
+    TileShared& S = tile_shared();
+    S.K.set(P, L.grid != 0);
+    S.w = P.w;
+    S.h = P.h;
+    S.x0 = (tile % P.tiles_x) * L.tw;
+    S.y0 = (tile / P.tiles_x) * L.th;
+    S.x1 = min(S.x0 + L.tw, P.w);
+    S.y1 = min(S.y0 + L.th, P.h);
+    S.lx0 = max(S.x0 - kHaloPerIter, 0);
+    S.ly0 = max(S.y0 - kHaloPerIter, 0);
+    S.RW = min(S.x1 + kHaloPerIter, P.w) - S.lx0;
+    S.RH = min(S.y1 + kHaloPerIter, P.h) - S.ly0;
 }
 
 // Persistent launch: each CTA takes tiles from the launch's queue (an atomic counter, zeroed before the launch)
 // until it is empty, so the last wave has no idle tail.  queue[i] = (problem index, tile index in problem).
-// Instantiated for 128, 256 and 512 threads, with and without speculative random-candidate loads, per cost, for
-// levels and for sub-scale grids (GRID).
-template <int THREADS, bool SPEC, class C, bool GRID = false>
-__global__ __launch_bounds__(THREADS, SPEC ? 1 : 512 / THREADS) void k_propagate(
+// Instantiated for 128, 256 and 512 threads, per cost (direct variant).
+template <int THREADS, class C>
+__global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
     PropLaunch L) {
     grid_dependency_sync();
-    extern __shared__ uint32_t smem[];
     __shared__ int s_next;
     for (;;) {
         if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
@@ -410,7 +874,9 @@ __global__ __launch_bounds__(THREADS, SPEC ? 1 : 512 / THREADS) void k_propagate
         const int q = s_next;
         if (q >= n_tiles) return;
         const int2 e = queue[q];
-        propagate_tile<C, SPEC, GRID>(probs[e.x], e.y, L, smem);
+        const PropProblem& P = probs[e.x];
+        const TileIO io = {P.flow_in, P.cost_in, P.flow_out, P.cost_out, P.t0, P.n_iter};
+        propagate_tile_direct<C, false>(P, e.y, L, g_smem, io);
         __syncthreads();
     }
 }
@@ -439,12 +905,11 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <int THREADS, bool SPEC, class C, bool GRID = false>
-__global__ __launch_bounds__(THREADS, SPEC ? 1 : 512 / THREADS) void k_propagate_df(
+template <int THREADS, class C, bool LISTED>
+__global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_propagate_df(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
-    PropLaunch L) {
+    PropLaunch L, TileLayout LT) {
     grid_dependency_sync();
-    extern __shared__ uint32_t smem[];
     __shared__ int s_next;
     const int T = L.dataflow, n_tasks = n_tiles * T;
     bool failed = false;  // a wait of this CTA expired: stop waiting (CTA-uniform)
@@ -466,6 +931,13 @@ __global__ __launch_bounds__(THREADS, SPEC ? 1 : 512 / THREADS) void k_propagate
         const int t = q / n_tiles;
         const int2 e = queue[q - t * n_tiles];
         const PropProblem& P = probs[e.x];
+        const bool src_alt = t > 0 && ((t - 1) & 1) == 0;  // iteration t - 1 wrote flow_alt iff t - 1 is even
+        const bool dst_alt = (t & 1) == 0;
+        const TileIO io = {src_alt ? P.flow_alt : P.flow_in, src_alt ? P.cost_alt : P.cost_in,
+                           t == T - 1 ? P.flow_out : dst_alt ? P.flow_alt : P.flow_in,
+                           t == T - 1 ? P.cost_out : dst_alt ? P.cost_alt : P.cost_in, P.t0 + t, 1};
+        if constexpr (LISTED)
+            if (threadIdx.x == 32) tile_setup(P, e.y, L), tile_shared().io = io;
         bool ok = true;
         if (t > 0 && !failed && threadIdx.x < 9) {  // one waiting thread per tile of the 3x3 neighbourhood
             const int tiles_y = (P.h + L.th - 1) / L.th;
@@ -481,15 +953,10 @@ __global__ __launch_bounds__(THREADS, SPEC ? 1 : 512 / THREADS) void k_propagate
             }
         }
         failed = __syncthreads_or(!ok) != 0 || failed;
-        TileIO io;
-        io.t0 = P.t0 + t;
-        io.n_iter = 1;
-        const bool src_alt = t > 0 && ((t - 1) & 1) == 0;  // iteration t - 1 wrote flow_alt iff t - 1 is even
-        io.flow_in = t == 0 ? P.flow_in : src_alt ? P.flow_alt : P.flow_in;
-        io.cost_in = t == 0 ? P.cost_in : src_alt ? P.cost_alt : P.cost_in;
-        io.flow_out = t == T - 1 ? P.flow_out : (t & 1) == 0 ? P.flow_alt : P.flow_in;
-        io.cost_out = t == T - 1 ? P.cost_out : (t & 1) == 0 ? P.cost_alt : P.cost_in;
-        propagate_tile<C, SPEC, GRID, true>(P, e.y, L, smem, &io);
+        if constexpr (LISTED)
+            propagate_tile_listed<C, THREADS>(P, LT);
+        else
+            propagate_tile_direct<C, true>(P, e.y, L, g_smem, io);
         __syncthreads();  // every store of the tile is issued
         if (threadIdx.x == 0 && !L.withhold) {
             __threadfence();
@@ -544,11 +1011,10 @@ __device__ __forceinline__ int colour_count(int k, int a, int b, int c) {
     return first < b ? (b - 1 - first) / 2 + 1 : 0;
 }
 
-// (no speculative variant: measured slower at every coarse level in this form)
-template <int THREADS, class C, bool GRID = false>
+template <int THREADS, class C>
 __global__ __launch_bounds__(THREADS, 1) void k_propagate_cl(const PropProblem* __restrict__ probs, PropLaunch L) {
     grid_dependency_sync();
-    extern __shared__ __align__(16) uint32_t smem[];
+    uint32_t* smem = g_smem;
     const int n = cluster_ctas(), r = cluster_rank();
     const PropProblem& P = probs[blockIdx.x / n];
     const int w = P.w, h = P.h;
@@ -611,7 +1077,7 @@ __global__ __launch_bounds__(THREADS, 1) void k_propagate_cl(const PropProblem* 
     }
     cluster_sync_all();  // every CTA of the cluster running, its block loaded and its mbarriers armed
     const int HW = (bw + 1) >> 1, total = HW * bh;
-    const SweepConst K = sweep_const<GRID>(P);
+    const SweepConst K = sweep_const(P, L.grid != 0);
     bool failed = false;  // a wait expired: stop waiting (CTA-uniform)
     uint32_t k1 = 0;
     for (int j = 0; j < J; j++) {
@@ -650,7 +1116,7 @@ __global__ __launch_bounds__(THREADS, 1) void k_propagate_cl(const PropProblem* 
                 else
                     f2 = sflow[sidx + (n2y - y) * bw];
             }
-            if (update_pixel<C, false, GRID>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) {
+            if (update_direct<C>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) {
                 sflow[sidx] = cur;
                 scost[sidx] = c;
             }
@@ -686,51 +1152,32 @@ __global__ __launch_bounds__(THREADS, 1) void k_propagate_cl(const PropProblem* 
 using PropKernel = void (*)(const PropProblem*, const int2*, int, int*, PropLaunch);
 using PropClusterKernel = void (*)(const PropProblem*, PropLaunch);
 
-template <class C, bool SPEC, bool GRID>
+using PropDataflowKernel = void (*)(const PropProblem*, const int2*, int, int*, PropLaunch, TileLayout);
+
+template <class C>
 PropKernel prop_kernel_t(int threads) {
-    return threads == 128   ? k_propagate<128, SPEC, C, GRID>
-           : threads == 512 ? k_propagate<512, SPEC, C, GRID>
-                            : k_propagate<256, SPEC, C, GRID>;
+    return threads == 128 ? k_propagate<128, C> : threads == 512 ? k_propagate<512, C> : k_propagate<256, C>;
+}
+PropKernel prop_kernel(int threads, int cost) {
+    return cost == FF_COST_CENSUS ? prop_kernel_t<CostCensus>(threads) : prop_kernel_t<CostSad>(threads);
 }
 
+// The direct variant is instantiated for 128, 256 and 512 threads, the listed one for 256 and 512 (prop_listed).
 template <class C>
-PropKernel prop_kernel_c(int threads, bool spec, bool grid) {
-    if (grid) return spec ? prop_kernel_t<C, true, true>(threads) : prop_kernel_t<C, false, true>(threads);
-    return spec ? prop_kernel_t<C, true, false>(threads) : prop_kernel_t<C, false, false>(threads);
+PropDataflowKernel prop_df_kernel_t(int threads, bool listed) {
+    if (listed) return threads == 512 ? k_propagate_df<512, C, true> : k_propagate_df<256, C, true>;
+    return threads == 128   ? k_propagate_df<128, C, false>
+           : threads == 512 ? k_propagate_df<512, C, false>
+                            : k_propagate_df<256, C, false>;
+}
+PropDataflowKernel prop_df_kernel(int threads, int cost, bool listed) {
+    return cost == FF_COST_CENSUS ? prop_df_kernel_t<CostCensus>(threads, listed) : prop_df_kernel_t<CostSad>(threads, listed);
 }
 
-PropKernel prop_kernel(int threads, bool spec, int cost, bool grid = false) {
-    return cost == FF_COST_CENSUS ? prop_kernel_c<CostCensus>(threads, spec, grid)
-                                  : prop_kernel_c<CostSad>(threads, spec, grid);
-}
-
-// The dataflow form is instantiated for 128, 256 and 512 threads without speculation, per cost, for levels and
-// for sub-scale grids.
-template <class C, bool GRID>
-PropKernel prop_df_kernel_t(int threads) {
-    return threads == 128   ? k_propagate_df<128, false, C, GRID>
-           : threads == 512 ? k_propagate_df<512, false, C, GRID>
-                            : k_propagate_df<256, false, C, GRID>;
-}
-
-PropKernel prop_df_kernel(int threads, int cost, bool grid) {
-    if (cost == FF_COST_CENSUS) return grid ? prop_df_kernel_t<CostCensus, true>(threads) : prop_df_kernel_t<CostCensus, false>(threads);
-    return grid ? prop_df_kernel_t<CostSad, true>(threads) : prop_df_kernel_t<CostSad, false>(threads);
-}
-
-// The cluster form is instantiated for 256 and 512 threads, per cost, for levels and for sub-scale grids.
-template <class C, bool GRID>
-PropClusterKernel prop_cl_kernel_t(int threads) {
-    return threads == 512 ? k_propagate_cl<512, C, GRID> : k_propagate_cl<256, C, GRID>;
-}
-
-template <class C>
-PropClusterKernel prop_cl_kernel_c(int threads, bool grid) {
-    return grid ? prop_cl_kernel_t<C, true>(threads) : prop_cl_kernel_t<C, false>(threads);
-}
-
-PropClusterKernel prop_cl_kernel(int threads, int cost, bool grid) {
-    return cost == FF_COST_CENSUS ? prop_cl_kernel_c<CostCensus>(threads, grid) : prop_cl_kernel_c<CostSad>(threads, grid);
+// The cluster form is instantiated for 256 and 512 threads, per cost.
+PropClusterKernel prop_cl_kernel(int threads, int cost) {
+    if (cost == FF_COST_CENSUS) return threads == 512 ? k_propagate_cl<512, CostCensus> : k_propagate_cl<256, CostCensus>;
+    return threads == 512 ? k_propagate_cl<512, CostSad> : k_propagate_cl<256, CostSad>;
 }
 
 cudaLaunchConfig_t cluster_config(int n_ctas, int cluster, int threads, size_t smem, cudaStream_t st,
@@ -756,48 +1203,46 @@ cudaError_t init_kernel_attributes() {
     cudaError_t e0 = cudaFuncGetAttributes(&fa, k_handover<CostSad>);
     if (e0 == cudaSuccess) e0 = cudaFuncGetAttributes(&fa, k_handover<CostCensus>);
     if (e0 != cudaSuccess) return e0;
-    for (int cost : {FF_COST_WHT_SAD, FF_COST_CENSUS})
-        for (int t : {128, 256, 512})
-            for (bool sp : {false, true})
-                for (bool grid : {false, true}) {
-                    cudaError_t e = cudaFuncSetAttribute(prop_kernel(t, sp, cost, grid),
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)kMaxPropSmem);
-                    if (e == cudaSuccess && !sp)
-                        e = cudaFuncSetAttribute(prop_df_kernel(t, cost, grid),
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPropSmem);
-                    if (e != cudaSuccess) return e;
-                }
-    for (int cost : {FF_COST_WHT_SAD, FF_COST_CENSUS})
-        for (int t : {256, 512})
-            for (bool grid : {false, true}) {
-                PropClusterKernel k = prop_cl_kernel(t, cost, grid);
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPropSmem);
-                if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int cost : {FF_COST_WHT_SAD, FF_COST_CENSUS}) {
+        for (int t : {128, 256, 512}) {
+            const void* ks[3] = {reinterpret_cast<const void*>(prop_kernel(t, cost)),
+                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, false)),
+                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, true))};
+            for (int v = 0; v < 3; v++) {
+                cudaError_t e = cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)(v == 2 ? kMaxTileSmem : kMaxPropSmem));
                 if (e != cudaSuccess) return e;
             }
+        }
+        for (int t : {256, 512}) {
+            PropClusterKernel k = prop_cl_kernel(t, cost);
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPropSmem);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+    }
     return cudaSuccess;
 }
 
 bool prop_threads_ok(int threads) { return threads == 128 || threads == 256 || threads == 512; }
 
-int prop_blocks_per_sm(size_t smem, int threads, bool spec, int cost, bool grid, bool dataflow) {
+int prop_blocks_per_sm(size_t smem, int threads, int cost, bool dataflow, bool listed) {
     int n = 0;
-    PropKernel k = dataflow ? prop_df_kernel(threads, cost, grid) : prop_kernel(threads, spec, cost, grid);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) !=
-        cudaSuccess) {
+    const void* k = dataflow ? reinterpret_cast<const void*>(prop_df_kernel(threads, cost, listed))
+                             : reinterpret_cast<const void*>(prop_kernel(threads, cost));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
     return n > 0 ? n : 1;
 }
 
-int prop_cluster_capacity(int cluster, int threads, int cost, bool grid, size_t smem) {
+int prop_cluster_capacity(int cluster, int threads, int cost, size_t smem) {
     if (cluster < 1 || cluster > kMaxCluster || (threads != 256 && threads != 512) || smem > kMaxPropSmem) return 0;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = cluster_config(cluster, cluster, threads, smem, nullptr, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, prop_cl_kernel(threads, cost, grid), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, prop_cl_kernel(threads, cost), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -809,13 +1254,16 @@ void launch_propagate(const PropProblem* probs_dev, const int2* queue_dev, int n
     if (L.cluster > 0) {
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = cluster_config(grid, L.cluster, L.threads, (size_t)L.cl_smem, st, attr);
-        cudaLaunchKernelEx(&cfg, prop_cl_kernel(L.threads, L.cost, L.grid != 0), probs_dev, L);
+        cudaLaunchKernelEx(&cfg, prop_cl_kernel(L.threads, L.cost), probs_dev, L);
         return;
     }
-    size_t smem = prop_smem_bytes(L.tw, L.th, L.max_iter);
-    PropKernel k = L.dataflow > 0 ? prop_df_kernel(L.threads, L.cost, L.grid != 0)
-                                  : prop_kernel(L.threads, L.spec != 0, L.cost, L.grid != 0);
-    launch_k(k, dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles, counter_dev, L);
+    const size_t smem = prop_launch_smem(L.tw, L.th, L.max_iter, L.listed != 0);
+    if (L.dataflow > 0)
+        launch_k(prop_df_kernel(L.threads, L.cost, L.listed != 0), dim3(grid), dim3(L.threads), smem, st, probs_dev,
+                 queue_dev, n_tiles, counter_dev, L, tile_layout(L.tw, L.th));
+    else
+        launch_k(prop_kernel(L.threads, L.cost), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles,
+                 counter_dev, L);
 }
 
 }  // namespace ff

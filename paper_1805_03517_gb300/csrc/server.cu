@@ -257,7 +257,7 @@ ff_status admit(ff_server* s) {
                 const TileChoice& t = q.cfg[l][g];
                 if (t.k < 1 || t.tw < 1 || t.th < 1 || !prop_threads_ok(t.threads) ||
                     prop_smem_bytes(t.tw, t.th, t.dataflow ? 1 : t.k) > kMaxPropSmem ||
-                    (t.dataflow && (t.tw < 4 || t.th < 4 || t.spec))) {
+                    (t.dataflow && (t.tw < 4 || t.th < 4))) {
                     st = srv_fail(s, FF_ERR_CUDA, "invalid launch configuration");
                     break;
                 }
@@ -279,10 +279,10 @@ ff_status admit(ff_server* s) {
 // Propagation launches of a tick are grouped by phase (the position of a chunk among the chunks one request
 // runs in this tick: a request's chunk i + 1 reads what its chunk i wrote) and by launch configuration.
 struct PropGroupKey {
-    int phase, tw, th, n_iter, threads, spec, grid, dataflow;
+    int phase, tw, th, n_iter, threads, grid, dataflow, listed;
     bool operator<(const PropGroupKey& o) const {
-        return std::tie(phase, tw, th, n_iter, threads, spec, grid, dataflow) <
-               std::tie(o.phase, o.tw, o.th, o.n_iter, o.threads, o.spec, o.grid, o.dataflow);
+        return std::tie(phase, tw, th, n_iter, threads, grid, dataflow, listed) <
+               std::tie(o.phase, o.tw, o.th, o.n_iter, o.threads, o.grid, o.dataflow, o.listed);
     }
 };
 
@@ -368,7 +368,7 @@ ff_status tick(ff_server* s) {
             const int chunk = q.chunk + phase;
             const int t0 = chunk * c.k, n_iter = std::min(c.k, T - t0);
             const bool last = sl == 0 && gk == 0 && chunk == q.n_chunks[sl][gk] - 1;
-            auto& grp = groups[PropGroupKey{phase, c.tw, c.th, n_iter, c.threads, c.spec, gk > 0 ? 1 : 0, c.dataflow}];
+            auto& grp = groups[PropGroupKey{phase, c.tw, c.th, n_iter, c.threads, gk > 0 ? 1 : 0, c.dataflow, c.listed}];
             for (int d = 0; d < 2; d++) {
                 const PyrView& X = d == 0 ? q.A : q.B;
                 const PyrView& Y = d == 0 ? q.B : q.A;
@@ -403,7 +403,8 @@ ff_status tick(ff_server* s) {
                 pp.level = sl + kMaxLevels * gk;  // the hash stream of this level or grid
                 pp.dir = d;
                 pp.seed = s->cv.seed;
-                pp.rs_radius = s->cv.rs_radius;
+                pp.rs_radius = (uint16_t)s->cv.rs_radius;
+                pp.T = (uint16_t)T;
                 grp.push_back({pp, pp.tiles_x * ((pp.h + c.th - 1) / c.th)});
             }
         }
@@ -477,11 +478,12 @@ ff_status tick(ff_server* s) {
             }
             pi++;
         }
-        const size_t smem = prop_smem_bytes(k.tw, k.th, k.dataflow ? 1 : k.n_iter);
+        const size_t smem = prop_launch_smem(k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.listed != 0);
         const int nq = (int)(qi - q0);
-        PropLaunch pl{k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.threads, k.spec, s->cv.cost, k.grid};
+        PropLaunch pl{k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.threads, s->cv.cost, k.grid};
+        pl.listed = k.listed;
         const int slots =
-            prop_blocks_per_sm(smem, k.threads, k.spec != 0, s->cv.cost, k.grid != 0, k.dataflow != 0) * s->cv.n_sms;
+            prop_blocks_per_sm(smem, k.threads, s->cv.cost, k.dataflow != 0, k.listed != 0) * s->cv.n_sms;
         if (k.dataflow) {
             pl.dataflow = k.n_iter;
             pl.affine = k.dataflow == 2;
