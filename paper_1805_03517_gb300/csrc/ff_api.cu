@@ -151,7 +151,7 @@ const TileCfg kCands[] = {
     {32, 16, 1, 128, 0}, {16, 16, 1, 128, 0}, {16, 8, 2, 128, 0},  {8, 8, 3, 128, 0},   {32, 32, 1, 512, 0},
     {32, 16, 2, 512, 0}, {16, 16, 2, 512, 0}, {24, 24, 1, 512, 0},
     // coarse levels: one pixel per thread per half-sweep (fewer dependent loads in a row)
-    {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},   {16, 16, 1, 512, 0}, {8, 8, 6, 512, 0},
+    {8, 4, 2, 256, 0},   {8, 4, 2, 512, 0},   {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},   {16, 16, 1, 512, 0}, {8, 8, 6, 512, 0},
     // fine levels: larger tiles recompute a smaller share of halo pixels
     {64, 32, 1, 128, 0}, {48, 32, 1, 128, 0}, {48, 32, 1, 256, 0}, {64, 16, 1, 128, 0}, {40, 24, 1, 128, 0},
     {48, 24, 1, 128, 0}, {64, 24, 1, 256, 0}, {64, 24, 1, 128, 0}, {96, 24, 1, 256, 0}, {80, 24, 1, 256, 0},
@@ -337,7 +337,7 @@ TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow
         if (level_pix_all > 50000) return {26, 16, 1, 512, 0, 0, 1};
         if (level_pix_all > 20000) return {16, 8, 1, 256, 0, 0, 1};
         if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
-        return {8, 8, std::min(2, T), 256, 0};
+        return {8, level_pix_all > 4000 ? 8 : 4, std::min(2, T), 256, 0};
     }
     // tile form only (a launch per group of iterations): large tiles with one iteration per launch when the level
     // fills the GPU, otherwise small tiles with fused iterations
@@ -347,7 +347,7 @@ TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow
     if (level_pix_all > 50000) return {16, 16, 1, 256, 0};
     if (level_pix_all > 20000) return {16, 8, 1, 256, 0};
     if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
-    return {8, 8, std::min(2, T), 256, 0};
+    return {8, level_pix_all > 4000 ? 8 : 4, std::min(2, T), 256, 0};
 }
 
 ff_status enqueue_launch(ff_ctx* c, const Launch& L) {

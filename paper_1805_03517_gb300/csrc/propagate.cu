@@ -223,75 +223,79 @@ struct TileGeom {
     int lx0, ly0, RW, RH;    // loaded region (tile + halo, clipped to the level)
 };
 
-// Region of half-sweep j (colour j&1 of direction j>>1) with `rem` halo pixels still to be consumed.
-__device__ __forceinline__ void halfsweep_region(const TileGeom& G, int w, int h, int j, int rem, int& rx0, int& ry0,
-                                                 int& rx1, int& ry1) {
-    rx0 = max(G.x0 - c_grow[j][0] - rem, 0);
-    ry0 = max(G.y0 - c_grow[j][1] - rem, 0);
-    rx1 = min(G.x1 + c_grow[j][2] + rem, w);
-    ry1 = min(G.y1 + c_grow[j][3] + rem, h);
-}
+// Regions of the half-sweeps of one iteration, in shared memory: x0, y0, x1, y1 in level coordinates, and
+// ceil(2^32 / slots per row), by which the index of a pixel of the active colour is divided.
+struct SweepRegions {
+    int4 r[8];
+    uint32_t inv[8];
+    // Thread j sets that of half-sweep j (colour j&1 of direction j>>1) with `rem` halo pixels still to be consumed.
+    __device__ __forceinline__ void set(const TileGeom& G, int w, int h, int rem) {
+        const int j = threadIdx.x;
+        if (j >= 8) return;
+        r[j] = make_int4(max(G.x0 - c_grow[j][0] - rem, 0), max(G.y0 - c_grow[j][1] - rem, 0),
+                         min(G.x1 + c_grow[j][2] + rem, w), min(G.y1 + c_grow[j][3] + rem, h));
+        inv[j] = 0xffffffffu / (uint32_t)((r[j].z - r[j].x + 1) >> 1) + 1u;  // (unused for one slot per row)
+    }
+};
 
-// Pixel i of the active colour of a region, row-major over (row, slot); false past the row's end.
-__device__ __forceinline__ bool region_pixel(int i, int HW, int rx0, int ry0, int rx1, int colour, int& x, int& y) {
-    const int row = i / HW, slot = i - row * HW;
-    y = ry0 + row;
-    x = rx0 + 2 * slot + ((rx0 + y + colour) & 1);
-    return x < rx1;
-}
-
-// Per-launch constants of update_direct, read from the problem once per half-sweep.
+// Per-launch constants of the pixel updates, read from the problem once per tile.
 struct SweepConst {
-    int g, lw, lh;  // grid stride and level size: grid pixel (x, y) is level pixel (g*x, g*y)
-    int R;          // random-search radius
-    uint32_t span;  // 2R + 1
+    const void* fa;
+    const void* fb;
+    int g, lw, lh;       // grid stride and level size: grid pixel (x, y) is level pixel (g*x, g*y)
+    int R;               // random-search radius
+    uint32_t span, inv;  // 2R + 1 and floor(2^32 / span)
+    // hash % span - R; the quotient is at most one too small
+    __device__ __forceinline__ int offset(uint32_t hash) const {
+        const uint32_t m = hash - __umulhi(hash, inv) * span;
+        return (int)(m >= span ? m - span : m) - R;
+    }
 };
 __device__ __forceinline__ SweepConst sweep_const(const PropProblem& P, bool grid) {
-    const int R = P.rs_radius;
-    return {grid ? P.g : 1, grid ? P.lw : P.w, grid ? P.lh : P.h, R, 2u * R + 1u};
+    const uint32_t span = 2u * P.rs_radius + 1u;
+    // (2^32 and 2^32 - 1 have the same quotient, except for span 1, where every offset is 0 anyway)
+    return {P.fa, P.fb, grid ? P.g : 1, grid ? P.lw : P.w, grid ? P.lh : P.h, P.rs_radius, span, 0xffffffffu / span};
 }
 
-// The candidates of one pixel (x, y) of a grid in a half-sweep of direction d, one thread per pixel (the whole
-// descriptor per thread: 96 B WHT, 32 B Census): neighbour 1 (horizontal, flow f1, valid if v1), neighbour 2
-// (vertical, f2, v2) and, for d >= 1, the hashed random offset around the flow after them.  cur / c hold the
-// pixel's flow and cost and are updated; false if there was nothing to try (they are unchanged).
+// The candidates of one pixel (x, y) of a grid in a half-sweep of direction d: neighbour 1 (horizontal, flow f1, valid
+// if v1), neighbour 2 (vertical, f2, v2) and, for d >= 1, the hashed random offset around the flow after them.  cur / c
+// hold the pixel's flow and cost and are updated; false if there was nothing to try (they are unchanged).  One thread
+// per pixel holds the whole descriptors.  (Four threads per pixel, one sector each, were slower at every level: 51
+// instead of 38 us already for the 32x24 level of the 128x96 pair.)
 template <class C>
-__device__ __forceinline__ bool update_direct(const PropProblem& P, const SweepConst& K, int x, int y, int d,
-                                              uint32_t k1, bool v1, uint32_t f1, bool v2, uint32_t f2, uint32_t& cur,
-                                              int& c) {
+__device__ __forceinline__ bool update_direct(const SweepConst& K, int x, int y, int d, uint32_t k1, bool v1, uint32_t f1,
+                                              bool v2, uint32_t f2, uint32_t& cur, int& c) {
     // flows and targets are in level pixels
-    const int g = K.g, lw = K.lw, lh = K.lh, R = K.R;
-    const uint32_t span = K.span;
+    const int g = K.g, lw = K.lw, lh = K.lh;
     const int n_d = lw * lh;  // descriptors of the level
     // a candidate equal to the current flow (or to an already tried one) cannot be strictly cheaper
     const int X = g * x, Y = g * y;  // level coordinates
     const bool e1 = v1 && f1 != cur && in_level(X + flow_x(f1), Y + flow_y(f1), lw, lh);
     const bool e2 = v2 && f2 != cur && !(v1 && f2 == f1) && in_level(X + flow_x(f2), Y + flow_y(f2), lw, lh);
     if (!(e1 || e2 || d >= 1)) return false;
+    // issue every independent load (own descriptor, neighbour candidates) before compute, the hash among them
+    uint32_t a[C::kSectors][8], b1[C::kSectors][8], b2[C::kSectors][8];
+    load_all<C>(K.fa, feat_index(X, Y, lw), n_d, kBoundsOwn, a);
+    if (e1) load_all<C>(K.fb, feat_index(X + flow_x(f1), Y + flow_y(f1), lw), n_d, kBoundsCand1, b1);
+    if (e2) load_all<C>(K.fb, feat_index(X + flow_x(f2), Y + flow_y(f2), lw), n_d, kBoundsCand2, b2);
     int ox = 0, oy = 0;
     if (d >= 1) {
         const uint32_t k2 = pixel_key(k1, X, Y);
-        ox = (int)(mix32(k2 ^ (uint32_t)(2 * d)) % span) - R;
-        oy = (int)(mix32(k2 ^ (uint32_t)(2 * d + 1)) % span) - R;
+        ox = K.offset(mix32(k2 ^ (uint32_t)(2 * d)));
+        oy = K.offset(mix32(k2 ^ (uint32_t)(2 * d + 1)));
     }
-    const bool rnd = ox != 0 || oy != 0;
-    // issue every independent load (own descriptor, neighbour candidates) before compute
-    uint32_t a[C::kSectors][8], b1[C::kSectors][8], b2[C::kSectors][8];
-    load_all<C>(P.fa, feat_index(X, Y, lw), n_d, kBoundsOwn, a);
-    if (e1) load_all<C>(P.fb, feat_index(X + flow_x(f1), Y + flow_y(f1), lw), n_d, kBoundsCand1, b1);
-    if (e2) load_all<C>(P.fb, feat_index(X + flow_x(f2), Y + flow_y(f2), lw), n_d, kBoundsCand2, b2);
     if (e1) {
-        int s1 = dist_all<C>(a, b1);
+        const int s1 = dist_all<C>(a, b1);
         if (s1 < c) { cur = f1; c = s1; }
     }
     if (e2) {
-        int s2 = dist_all<C>(a, b2);
+        const int s2 = dist_all<C>(a, b2);
         if (s2 < c) { cur = f2; c = s2; }
     }
-    if (rnd) {
+    if (ox != 0 || oy != 0) {
         const int fx = flow_x(cur) + ox, fy = flow_y(cur) + oy;
         if (in_level(X + fx, Y + fy, lw, lh)) {
-            load_all<C>(P.fb, feat_index(X + fx, Y + fy, lw), n_d, kBoundsRandom, b1);
+            load_all<C>(K.fb, feat_index(X + fx, Y + fy, lw), n_d, kBoundsRandom, b1);
             const int s3 = dist_all<C>(a, b1);
             if (s3 < c) { cur = pack_flow(fx, fy); c = s3; }
         }
@@ -301,18 +305,14 @@ __device__ __forceinline__ bool update_direct(const PropProblem& P, const SweepC
 
 // One half-sweep of a tile's region (direct variant).
 template <class C>
-__device__ __forceinline__ void halfsweep_direct(const PropProblem& P, const TileGeom& G, uint32_t* sflow,
-                                                 int32_t* scost, int j, int rem, uint32_t k1, bool grid) {
-    const int w = P.w, h = P.h;  // the grid (the level itself unless g > 1)
+__device__ __forceinline__ void halfsweep_direct(const SweepConst& K, const TileGeom& G, int w, int h, const int4 r,
+                                                 uint32_t inv, uint32_t* sflow, int32_t* scost, int j, uint32_t k1) {
     const int d = j >> 1, colour = j & 1;
-    int rx0, ry0, rx1, ry1;
-    halfsweep_region(G, w, h, j, rem, rx0, ry0, rx1, ry1);
-    const int HW = (rx1 - rx0 + 1) >> 1;
-    const int total = HW * (ry1 - ry0);
-    const SweepConst K = sweep_const(P, grid);
+    const int HW = (r.z - r.x + 1) >> 1, total = HW * (r.w - r.y);
     for (int i = threadIdx.x; i < total; i += blockDim.x) {
-        int x, y;
-        if (!region_pixel(i, HW, rx0, ry0, rx1, colour, x, y)) continue;
+        const int row = HW > 1 ? (int)__umulhi((uint32_t)i, inv) : i;  // i, HW < 2^15: i / HW
+        const int y = r.y + row, x = r.x + 2 * (i - row * HW) + ((r.x + y + colour) & 1);
+        if (x >= r.z) continue;
         const int sidx = (y - G.ly0) * G.RW + (x - G.lx0);
         const int n_s = G.RW * G.RH;  // shared-memory entries
         if (!idx_ok(g_bounds, kBoundsSmemOwn, sidx, n_s)) continue;
@@ -325,7 +325,7 @@ __device__ __forceinline__ void halfsweep_direct(const PropProblem& P, const Til
         const uint32_t f1 = v1 && idx_ok(g_bounds, kBoundsSmemN1, sidx + (n1x - x), n_s) ? sflow[sidx + (n1x - x)] : 0u;
         const uint32_t f2 =
             v2 && idx_ok(g_bounds, kBoundsSmemN2, sidx + (n2y - y) * G.RW, n_s) ? sflow[sidx + (n2y - y) * G.RW] : 0u;
-        if (!update_direct<C>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) continue;
+        if (!update_direct<C>(K, x, y, d, k1, v1, f1, v2, f2, cur, c)) continue;
         sflow[sidx] = cur;
         scost[sidx] = c;
     }
@@ -336,6 +336,7 @@ __device__ __forceinline__ void halfsweep_direct(const PropProblem& P, const Til
 template <class C, bool DF>
 __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int tile, const PropLaunch& L,
                                                       uint32_t* smem, const TileIO& io) {
+    __shared__ SweepRegions s_regions[2];  // of iterations it and it + 1
     const int w = P.w, h = P.h;
     const int n_iter = io.n_iter;
     TileGeom G;
@@ -350,6 +351,8 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
     G.RH = min(G.y1 + H, h) - G.ly0;
     uint32_t* sflow = smem;
     int32_t* scost = reinterpret_cast<int32_t*>(smem + G.RW * G.RH);
+    const SweepConst K = sweep_const(P, L.grid != 0);
+    s_regions[0].set(G, w, h, kHaloPerIter * (n_iter - 1));
 
     for (int i = threadIdx.x; i < G.RW * G.RH; i += blockDim.x) {
         int r = i / G.RW, c = i - r * G.RW;
@@ -362,11 +365,11 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
     }
     __syncthreads();
     for (int it = 0; it < n_iter; it++) {
-        const int t = io.t0 + it;
-        const int rem = kHaloPerIter * (n_iter - 1 - it);
-        const uint32_t k1 = iter_key(P, t);
+        const uint32_t k1 = iter_key(P, io.t0 + it);
+        const SweepRegions& S = s_regions[it & 1];
+        if (it + 1 < n_iter) s_regions[(it + 1) & 1].set(G, w, h, kHaloPerIter * (n_iter - 2 - it));
         for (int j = 0; j < 8; j++) {
-            halfsweep_direct<C>(P, G, sflow, scost, j, rem, k1, L.grid != 0);
+            halfsweep_direct<C>(K, G, w, h, S.r[j], S.inv[j], sflow, scost, j, k1);
             __syncthreads();
         }
     }
@@ -496,8 +499,9 @@ struct SweepRef {
 // (horizontal, flow f1, to be tried if t1), neighbour 2 (vertical, f2, t2) and, for d >= 1, the hashed random
 // offset around the flow after them.  The random candidate is scored if `rnd`, or if a neighbour was taken (else it
 // is known not to be cheaper).  cur / c hold the pixel's flow and cost and are updated.
-// (The descriptors are cleared where a load may be left out: a register that a predicated load may leave unwritten
-// stays reserved through every enclosing loop, which cost 30 to 50 registers a thread and half of the warps.)
+// Each candidate's three sectors are loaded together and one candidate after the other, so that a late half-sweep,
+// where a pixel has one candidate to try, waits for one gather (level 0 of the 1242x375 pair: 541 us; both neighbours
+// side by side, sector by sector, and the random candidate until its partial distance settles it: 565).
 template <class C>
 __device__ __forceinline__ void update_pixel(const SweepRef K, int x, int y, int d, uint32_t k1, bool t1, uint32_t f1,
                                              bool t2, uint32_t f2, bool rnd, uint32_t& cur, int& c) {
@@ -506,41 +510,30 @@ __device__ __forceinline__ void update_pixel(const SweepRef K, int x, int y, int
     // a candidate equal to the current flow (or to an already tried one) cannot be strictly cheaper
     const bool e1 = t1 && f1 != cur && K.inside(X + flow_x(f1), Y + flow_y(f1));
     const bool e2 = t2 && f2 != cur && !(t1 && f2 == f1) && K.inside(X + flow_x(f2), Y + flow_y(f2));
-    const int own = K.index(X, Y);
     const uint32_t cur0 = cur;
-    uint32_t a[C::kSectors][8] = {};  // the own descriptor, kept if the neighbours are scored
-    const bool nb = e1 || e2;
-    if (nb) {
-        const int i1 = e1 ? K.index(X + flow_x(f1), Y + flow_y(f1)) : 0;
-        const int i2 = e2 ? K.index(X + flow_x(f2), Y + flow_y(f2)) : 0;
-        int s1 = 0, s2 = 0;
-#pragma unroll
-        for (int k = 0; k < C::kSectors; k++) {
-            uint32_t b1[8] = {}, b2[8] = {};
-            load_chk<C>(K.fa(), own, n_d, kBoundsOwn, k, a[k]);
-            if (e1) load_chk<C>(K.fb(), i1, n_d, kBoundsCand1, k, b1);
-            if (e2) load_chk<C>(K.fb(), i2, n_d, kBoundsCand2, k, b2);
-            if (e1) s1 = C::dist(a[k], b1, s1);
-            if (e2) s2 = C::dist(a[k], b2, s2);
-        }
-        if (e1 && s1 < c) { cur = f1; c = s1; }
-        if (e2 && s2 < c) { cur = f2; c = s2; }
+    uint32_t a[C::kSectors][8];
+    load_all<C>(K.fa(), K.index(X, Y), n_d, kBoundsOwn, a);
+    if (e1 || e2) {
+        const uint32_t f = e1 ? f1 : f2;
+        uint32_t b[C::kSectors][8];
+        load_all<C>(K.fb(), K.index(X + flow_x(f), Y + flow_y(f)), n_d, kBoundsCand1, b);
+        const int s1 = dist_all<C>(a, b);
+        if (s1 < c) { cur = f; c = s1; }
+    }
+    if (e1 && e2) {
+        uint32_t b[C::kSectors][8];
+        load_all<C>(K.fb(), K.index(X + flow_x(f2), Y + flow_y(f2)), n_d, kBoundsCand2, b);
+        const int s2 = dist_all<C>(a, b);
+        if (s2 < c) { cur = f2; c = s2; }
     }
     if (d >= 1 && (rnd || cur != cur0)) {
         int ox, oy;
         K.random_offset(pixel_key(k1, X, Y), d, ox, oy);
         const int fx = flow_x(cur) + ox, fy = flow_y(cur) + oy;
         if ((ox != 0 || oy != 0) && K.inside(X + fx, Y + fy)) {
-            const int i3 = K.index(X + fx, Y + fy);
-            int s3 = 0;
-#pragma unroll
-            for (int k = 0; k < C::kSectors; k++)
-                if (s3 < c) {  // (a partial distance that reaches the cost settles it)
-                    uint32_t b[8];
-                    if (!nb) load_chk<C>(K.fa(), own, n_d, kBoundsOwn, k, a[k]);
-                    load_chk<C>(K.fb(), i3, n_d, kBoundsRandom, k, b);
-                    s3 = C::dist(a[k], b, s3);
-                }
+            uint32_t b[C::kSectors][8];
+            load_all<C>(K.fb(), K.index(X + fx, Y + fy), n_d, kBoundsRandom, b);
+            const int s3 = dist_all<C>(a, b);
             if (s3 < c) { cur = pack_flow(fx, fy); c = s3; }
         }
     }
@@ -1116,7 +1109,7 @@ __global__ __launch_bounds__(THREADS, 1) void k_propagate_cl(const PropProblem* 
                 else
                     f2 = sflow[sidx + (n2y - y) * bw];
             }
-            if (update_direct<C>(P, K, x, y, d, k1, v1, f1, v2, f2, cur, c)) {
+            if (update_direct<C>(K, x, y, d, k1, v1, f1, v2, f2, cur, c)) {
                 sflow[sidx] = cur;
                 scost[sidx] = c;
             }
