@@ -390,8 +390,8 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
 //
 // What bounds the direct variant at level 0 of the 1242x375 pair is gathers and instructions alike: 28.9 M sectors
 // and 59 M instructions per iteration, most of them for candidates that are known not to be cheaper, at 44 % of the
-// issue slots.  This variant loads 13 M sectors per iteration and runs 32 instead of 16 warps per SM: level 0 in 567
-// instead of 663 us (all six iterations), of the 1920x1080 pair in 1816 instead of 2760.
+// issue slots.  This variant loads 13 M sectors per iteration and runs 32 instead of 16 warps per SM: level 0 in 538
+// instead of 663 us (all six iterations), of the 1920x1080 pair in 1700 instead of 2760.
 
 // What a pixel still has to try, one byte per pixel in shared memory.  Costs only fall and
 // a candidate's cost is fixed, so a candidate that was not cheaper than a pixel's flow never becomes so: a
@@ -587,7 +587,7 @@ void prop_fit_tile(int& tw, int& th) {
 
 // The line between the variants, from both timed in their best tiles (all iterations of a pass, WHT-SAD, T = 6, us,
 // direct / listed): 167 k pixels 160 / 199, 232 k 235 / 250, 259 k 248 / 248, 346 k 297 / 293, 614 k 360 / 299, 932 k
-// 663 / 567, 1.04 M 708 / 551, 4.1 M 2760 / 1816, 5.6 M 3794 / 2800; Census 232 k 147 / 156, 614 k 266 / 217, 4.1 M 1649 /
+// 663 / 538, 1.04 M 708 / 535, 4.1 M 2760 / 1700, 5.6 M 3794 / 2800; Census 232 k 147 / 156, 614 k 266 / 217, 4.1 M 1649 /
 // 1050.  Below it a half-sweep's chain of dependent loads bounds a pass, not the amount of work, and the direct
 // variant's chain is the shorter one.  What does not suit the listed variant keeps the direct one: the tile form (one
 // 640x480 direction 795 us listed, 639 direct: a launch per iteration leaves the screening's tail exposed), 128 threads
@@ -624,23 +624,27 @@ __device__ __forceinline__ void mark_neighbours(uint32_t* todo, int b, int slots
 // every pixel of the tile, the candidates of directions 1..3 around its present flow are scored side by
 // side, sector by sector, each until its partial distance reaches the pixel's cost.  A candidate that reaches it is
 // not cheaper, and stays so while the pixel keeps its flow; the others (a few per cent) are flagged in the state word
-// and scored again in their half-sweep, as are those of pixels whose flow has changed by then.  So the own descriptor is loaded once per iteration instead of once per
-// direction, candidates of matched pixels are mostly dropped after one of their three sectors, three gathers are in
-// flight per thread, the half-sweeps are left with few pixels, and a tile screens its own pixels only: the flags of
-// its halo come with the state its neighbours wrote.
+// and scored again in their half-sweep, as are those of pixels whose flow has changed by then.  So the own descriptor is loaded
+// once per iteration instead of once per direction, candidates of matched pixels are mostly dropped after one of their
+// three sectors, three gathers are in flight per thread, the half-sweeps are left with few pixels, and a tile screens
+// its own pixels only: the flags of its halo come with the state its neighbours wrote.
+// What bounds it is L1 (a quarter to a third of a pass at level 0).  So both colours go row by row, not one colour
+// after the other: a 128-byte line holds parts of two pixels' descriptors, and the second finds it in L1 (level 0 of
+// the 1920x1080 pair 1700 us, 1770 colour by colour; of the 1242x375 pair 538, 543).  Within a row the columns of even
+// x come first; plain rows (1708, 538) and warps of 16x2, 8x4 and 4x8 pixels (1725, 1700, 1710; 540, 538, 540) are no
+// faster.
 template <class C, int THREADS>
-__device__ __forceinline__ void screen(const TileLayout T, int colour, const int4 r, uint32_t k1) {
+__device__ __forceinline__ void screen(const TileLayout T, const int4 r, uint32_t k1) {
     const int tid = (int)fresh(threadIdx.x);
-    const int HWr = (r.z - r.x + 1) >> 1, total = HWr * (r.w - r.y);
-    const uint32_t inv = 0xffffffffu / (uint32_t)HWr + 1u;  // ceil(2^32 / HWr): i / HWr = umulhi(i, inv) for i < 2^15
+    const int W = r.z - r.x, total = W * (r.w - r.y);
+    const uint32_t inv = 0xffffffffu / (uint32_t)W + 1u;  // ceil(2^32 / W): i / W = umulhi(i, inv) for i < 2^15
 #pragma unroll 1
     for (int i = tid; i < total; i += THREADS) {
         const int4 O = tile_origin();
         const SweepRef K = tile_sweep();
-        const int row = HWr > 1 ? (int)__umulhi((uint32_t)i, inv) : i;
-        const int ry = r.y + row;
-        const int rx = r.x + 2 * (i - row * HWr) + ((O.x + O.y + r.x + ry + colour) & 1);
-        if (rx >= r.z) continue;
+        const int row = W > 1 ? (int)__umulhi((uint32_t)i, inv) : i, k = i - row * W;
+        const int odd = (O.x + r.x) & 1, n_even = (W + 1 - odd) >> 1;  // columns of even x, then those of odd x
+        const int ry = r.y + row, rx = r.x + (k < n_even ? 2 * k + odd : 2 * (k - n_even) + 1 - odd);
         const int sidx = (ry << (T.slots + 1)) + rx;
         if (!idx_ok(g_bounds, kBoundsSmemOwn, sidx, T.n_pixels())) continue;
         const uint32_t cur = g_smem[kHeadWords + sidx];
@@ -816,8 +820,7 @@ __device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, cons
     for (int j = 0; j < 8; j++) halfsweep<C, THREADS>(T, j, k1);
     if (!plain) {
         const uint32_t kn = iter_key(P, t + 1);
-#pragma unroll 1
-        for (int colour = 0; colour < 2; colour++) screen<C, THREADS>(T, colour, S.rect[7], kn);  // the tile
+        screen<C, THREADS>(T, S.rect[7], kn);  // of the tile
     }
     __syncthreads();
     const int TW = S.x1 - S.x0, n_out = TW * (S.y1 - S.y0);
