@@ -319,8 +319,8 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
 // pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both costs.  Passes the listed
 // variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the largest that leave the
 // queue more tiles than the 608 CTAs an SM's 2048 threads make (a Census distance is a third of the work, so larger
-// tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 538, 223, 110, 79 and 64 instead of 844, 375, 294, 113
-// and 75 with the rule for the tile form below; of the 1920x1080 pair 1705, 535, 243, 114 and 77 instead of 3280, 935,
+// tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 531, 221, 109, 77 and 61 instead of 844, 375, 294, 113
+// and 75 with the rule for the tile form below; of the 1920x1080 pair 1674, 527, 240, 113 and 76 instead of 3280, 935,
 // 594, 475 and 142.
 TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow_ok) {
     if (dataflow_ok) {

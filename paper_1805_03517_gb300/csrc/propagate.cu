@@ -390,8 +390,8 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
 //
 // What bounds the direct variant at level 0 of the 1242x375 pair is gathers and instructions alike: 28.9 M sectors
 // and 59 M instructions per iteration, most of them for candidates that are known not to be cheaper, at 44 % of the
-// issue slots.  This variant loads 13 M sectors per iteration and runs 32 instead of 16 warps per SM: level 0 in 538
-// instead of 663 us (all six iterations), of the 1920x1080 pair in 1700 instead of 2760.
+// issue slots.  This variant loads 13 M sectors per iteration and runs 32 instead of 16 warps per SM: level 0 in 531
+// instead of 663 us (all six iterations), of the 1920x1080 pair in 1674 instead of 2760.
 
 // What a pixel still has to try, one byte per pixel in shared memory.  Costs only fall and
 // a candidate's cost is fixed, so a candidate that was not cheaper than a pixel's flow never becomes so: a
@@ -587,7 +587,7 @@ void prop_fit_tile(int& tw, int& th) {
 
 // The line between the variants, from both timed in their best tiles (all iterations of a pass, WHT-SAD, T = 6, us,
 // direct / listed): 167 k pixels 160 / 199, 232 k 235 / 250, 259 k 248 / 248, 346 k 297 / 293, 614 k 360 / 299, 932 k
-// 663 / 538, 1.04 M 708 / 535, 4.1 M 2760 / 1700, 5.6 M 3794 / 2800; Census 232 k 147 / 156, 614 k 266 / 217, 4.1 M 1649 /
+// 663 / 531, 1.04 M 708 / 527, 4.1 M 2760 / 1674, 5.6 M 3794 / 2800; Census 232 k 147 / 156, 614 k 266 / 217, 4.1 M 1649 /
 // 1050.  Below it a half-sweep's chain of dependent loads bounds a pass, not the amount of work, and the direct
 // variant's chain is the shorter one.  What does not suit the listed variant keeps the direct one: the tile form (one
 // 640x480 direction 795 us listed, 639 direct: a launch per iteration leaves the screening's tail exposed), 128 threads
@@ -772,8 +772,9 @@ __device__ __forceinline__ void set_regions() {
 // One tile of one problem: load the tile and its halo, run iteration io.t0 in shared memory, write the tile.  The state
 // was written by other CTAs of the running launch and is therefore read from L2.  Between the tasks of a pass the cost buffers hold state words; a pass starts from plain costs and its last
 // iteration leaves plain costs.  The head of the shared memory is set (tile_setup).
+// With a counter, the CTA's next task is taken while this one is written, into *s_next.
 template <class C, int THREADS>
-__device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, const TileLayout T) {
+__device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, const TileLayout T, int* counter, int* s_next) {
     TileShared& S = tile_shared();
     {
         uint32_t* todo = g_smem + T.o_todo();
@@ -823,6 +824,8 @@ __device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, cons
         screen<C, THREADS>(T, S.rect[7], kn);  // of the tile
     }
     __syncthreads();
+    int next = 0;
+    if (counter && threadIdx.x == 0) next = atomicAdd(counter, 1);
     const int TW = S.x1 - S.x0, n_out = TW * (S.y1 - S.y0);
     const uint32_t inv = 0xffffffffu / (uint32_t)TW + 1u;
 #pragma unroll 1
@@ -837,6 +840,7 @@ __device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, cons
         const uint32_t st = g_smem[T.o_state() + sidx];
         S.io.cost_out[g] = (int32_t)(plain ? st >> kCostShift : st);
     }
+    if (counter && threadIdx.x == 0) *s_next = next;
 }
 
 // Problem and geometry of the CTA's next tile, by one thread.
@@ -855,8 +859,11 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
     S.RH = min(S.y1 + kHaloPerIter, P.h) - S.ly0;
 }
 
-// Persistent launch: each CTA takes tiles from the launch's queue (an atomic counter, zeroed before the launch)
-// until it is empty, so the last wave has no idle tail.  queue[i] = (problem index, tile index in problem).
+// Persistent launch: each CTA takes tiles from the launch's queue until it is empty, so the last wave has no idle tail.
+// CTA b starts with entry b; the others are taken with an atomic counter (zeroed before the launch) while the tile
+// before is worked on, and a launch with a CTA per tile takes none.  At small levels a launch is a chain of memory
+// round trips, of which this leaves out two (level 4 of the 1242x375 pair 64 -> 61 us, level 3 79 -> 77; the three
+// launches of the 32x24 level of the 128x96 pair 61 -> 58).  queue[i] = (problem index, tile index in problem).
 // Instantiated for 128, 256 and 512 threads, per cost (direct variant).
 template <int THREADS, class C>
 __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
@@ -864,15 +871,16 @@ __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
     PropLaunch L) {
     grid_dependency_sync();
     __shared__ int s_next;
-    for (;;) {
-        if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
-        __syncthreads();
-        const int q = s_next;
-        if (q >= n_tiles) return;
+    const int G = (int)gridDim.x;
+    for (int q = (int)blockIdx.x; q < n_tiles; q = s_next) {
+        int next = n_tiles;
+        if (G < n_tiles && threadIdx.x == 0) next = G + atomicAdd(counter, 1);
         const int2 e = queue[q];
         const PropProblem& P = probs[e.x];
         const TileIO io = {P.flow_in, P.cost_in, P.flow_out, P.cost_out, P.t0, P.n_iter};
         propagate_tile_direct<C, false>(P, e.y, L, g_smem, io);
+        if (G >= n_tiles) return;
+        if (threadIdx.x == 0) s_next = next;
         __syncthreads();
     }
 }
@@ -888,6 +896,11 @@ __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
 // a release after the tile's stores and read with an acquire; the region is then read from L2.  A task waits
 // only for tasks taken before it by running CTAs, so there is no deadlock whatever the residency; every wait is
 // bounded (wait_limit polls; on expiry kErrDataflow goes to the error word and the CTA stops waiting).
+// The round trips between two tasks overlap where they may: a warp that neither takes tasks nor polls publishes the
+// finished one, and the listed variant takes its next task while it writes the present one (which waits for nothing any
+// more, so the argument above holds): level 0 of the 1242x375 pair 538 -> 531 us, of the 1920x1080 pair 1700 -> 1674
+// (with Census 290 -> 294).  A task taken at the start of the one before is held too long (682, 1855), and in the
+// direct variant, with a tile or two per CTA and iteration, even one taken that late is (level 2: 109 -> 113).
 // Affine variant (L.affine): no queue counter; CTA b owns entries b, b + G, ... of every iteration (G CTAs, at
 // most the resident ones) and runs them iteration by iteration, keeping its tiles' descriptors in its L1.  Its
 // waits are for iteration t - 1 of tiles other CTAs own, which wait only for earlier iterations, so every CTA
@@ -919,8 +932,10 @@ __global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_pr
             const int ti = k / per_iter;
             q = ti * n_tiles + (int)blockIdx.x + (k - ti * per_iter) * G;
         } else {
-            if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
-            __syncthreads();
+            if (!LISTED || k == 0) {
+                if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
+                __syncthreads();
+            }
             q = s_next;
             if (q >= n_tasks) return;
         }
@@ -950,11 +965,11 @@ __global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_pr
         }
         failed = __syncthreads_or(!ok) != 0 || failed;
         if constexpr (LISTED)
-            propagate_tile_listed<C, THREADS>(P, LT);
+            propagate_tile_listed<C, THREADS>(P, LT, L.affine ? nullptr : counter, &s_next);
         else
             propagate_tile_direct<C, true>(P, e.y, L, g_smem, io);
         __syncthreads();  // every store of the tile is issued
-        if (threadIdx.x == 0 && !L.withhold) {
+        if (threadIdx.x == 64 && !L.withhold) {
             __threadfence();
             st_release_gpu(P.progress + e.y, t + 1);
         }
