@@ -313,15 +313,16 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
 }
 
 // Default propagation configuration of a pass that has not been tuned, by its pixels (all problems of its launches):
-// from 20,000 pixels the queue variant of the dataflow form (every iteration in one launch, no resident grid needed),
+// from 28,000 pixels the queue variant of the dataflow form (every iteration in one launch, no resident grid needed),
 // in tiles small enough to keep every SM busy; below, where a pass is a chain of half-sweeps on a few SMs, the tile
-// form with two iterations per launch, whose halo idle SMs absorb.  The lines are the near-best of a sweep over single
-// pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both costs.  Passes the listed
-// variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the largest that leave the
-// queue more tiles than the 608 CTAs an SM's 2048 threads make (a Census distance is a third of the work, so larger
-// tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 531, 221, 109, 77 and 61 instead of 844, 375, 294, 113
-// and 75 with the rule for the tile form below; of the 1920x1080 pair 1674, 527, 240, 113 and 76 instead of 3280, 935,
-// 594, 475 and 142.
+// form in tiles the resident variant takes (prop_resident, with its times), the largest that leave no second tile to
+// a CTA, and below 4,000 pixels with two iterations per launch, whose halo idle SMs absorb.  The lines are the near-best
+// of a sweep over single pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both
+// costs.  Passes the listed variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the
+// largest that leave the queue more tiles than the 608 CTAs an SM's 2048 threads make (a Census distance is a third of
+// the work, so larger tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 531, 221, 109, 72 and 50 instead of
+// 844, 375, 294, 113 and 75 with the rule before these variants; of the 1920x1080 pair 1674, 527, 240, 113 and 67
+// instead of 3280, 935, 594, 475 and 142.
 TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow_ok) {
     if (dataflow_ok) {
         if (prop_listed(level_pix_all, 56, 256, true)) {
@@ -335,19 +336,19 @@ TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow
         if (level_pix_all > 130000) return {24, 16, 1, 256, 0, 0, 1};
         if (level_pix_all > 75000) return {20, 12, 1, 256, 0, 0, 1};
         if (level_pix_all > 50000) return {26, 16, 1, 512, 0, 0, 1};
-        if (level_pix_all > 20000) return {16, 8, 1, 256, 0, 0, 1};
-        if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
-        return {8, level_pix_all > 4000 ? 8 : 4, std::min(2, T), 256, 0};
+        if (level_pix_all > 40000) return {16, 8, 1, 256, 0, 0, 1};
+        if (level_pix_all > 28000) return {16, 12, 1, 512, 0, 0, 1};
     }
+    if (level_pix_all <= 4000) return {8, 4, std::min(2, T), 512, 0};
+    if (level_pix_all <= 20000) return {8, 8, 1, 256, 0};
+    if (level_pix_all <= 28000) return {16, 12, 1, 512, 0};
     // tile form only (a launch per group of iterations): large tiles with one iteration per launch when the level
     // fills the GPU, otherwise small tiles with fused iterations
     const int64_t slots = (int64_t)c->n_sms * 2;
     if (level_pix_all / (32 * 32) >= 2 * slots) return {32, 32, 1, 256, 0};
     if (level_pix_all / (32 * 16) >= 2 * slots) return {32, 16, 1, 256, 0};
     if (level_pix_all > 50000) return {16, 16, 1, 256, 0};
-    if (level_pix_all > 20000) return {16, 8, 1, 256, 0};
-    if (level_pix_all > 8000) return {16, 8, std::min(2, T), 512, 0};
-    return {8, level_pix_all > 4000 ? 8 : 4, std::min(2, T), 256, 0};
+    return {16, 8, 1, 256, 0};
 }
 
 ff_status enqueue_launch(ff_ctx* c, const Launch& L) {

@@ -206,6 +206,10 @@ __device__ __forceinline__ uint32_t pixel_key(uint32_t k1, int X, int Y) {
     return mix32(k1 ^ ((uint32_t)Y * 65536u + (uint32_t)X));
 }
 
+// The variants of a tile's work: one pixel of a half-sweep at a time per thread, every pixel of the region by its own
+// thread, and lists of the pixels with something to try.
+enum Variant { kDirect, kResident, kListed };
+
 // Where a tile task reads the state of its region and writes its interior, and which iterations it runs.
 struct TileIO {
     const uint32_t* flow_in;
@@ -331,9 +335,122 @@ __device__ __forceinline__ void halfsweep_direct(const SweepConst& K, const Tile
     }
 }
 
+// ---- resident variant: a region of at most one pixel per thread
+//
+// A small level is a chain of half-sweeps, and a half-sweep one of a thread's instructions and gathers: of a warp's time
+// at level 4 of the 1242x375 pair, 42 % is issuing, 41 % waiting for gathers, and a half-sweep takes about a
+// microsecond whether the region has 60 or 170 pixels of its colour.  So every pixel of the region has a thread that
+// keeps its flow, cost and own descriptor in registers for all iterations of the launch (half the threads have the
+// pixels of one colour, half those of the other), which leaves three things off the chain.  A neighbour is tried only
+// if its flow is not the one tried last on that side (a candidate that was not cheaper never becomes so).  The random
+// candidate around the present flow, known before the half-sweep, is scored during the half-sweep of the other colour,
+// when the thread has nothing else to do; only a pixel that takes a neighbour's flow scores another one after it.  And
+// there is no index arithmetic.  Pass times (6 iterations, us) of the best tiles with / without, by pixels: WHT-SAD 96
+// 34 / 50, 1.5 k 54 / 58, 3.7 k 50 / 61, 10 k 68 / 78, 16 k 67 / 77, 25 k 82 / 94, 38 k 88 / 94, 42 k 102 / 98; Census
+// 33 / 43, 42 / 48, 45 / 50, 52 / 52, 57 / 53, 60 / 70, 72 / 74, 85 / 74.  (A pair of pixels per thread, one of each
+// colour and no thread idle, nor anything scored ahead: 90 instead of 61 at 3.7 k, spills included.)
+
+// Cost of the flow (fx, fy) of level pixel (X, Y) with descriptor a, INT_MAX if its target is outside the level.
+// (The arrays of predicated loads are zeroed, here and below: left uninitialised, they stay live around the loops and
+// the kernel spills.)
+template <class C>
+__device__ __forceinline__ int score(const SweepConst& K, int X, int Y, const uint32_t (&a)[C::kSectors][8], int fx, int fy) {
+    if (!in_level(X + fx, Y + fy, K.lw, K.lh)) return INT_MAX;
+    uint32_t b[C::kSectors][8] = {};
+    load_all<C>(K.fb, feat_index(X + fx, Y + fy, K.lw), K.lw * K.lh, kBoundsRandom, b);
+    return dist_all<C>(a, b);
+}
+
+// One tile of one problem, as propagate_tile_direct, whose geometry and regions it takes.  The flows are in shared
+// memory by colour: pixel (rx, ry) of the region has slot ry * ceil(RW / 2) + rx / 2 of its colour.
+template <class C, bool DF>
+__device__ __forceinline__ void propagate_tile_resident(const SweepConst& K, const TileGeom& G, const PropProblem& P,
+                                                        uint32_t* smem, const TileIO& io, SweepRegions* s_regions) {
+    const int w = P.w, h = P.h, n_iter = io.n_iter;
+    const int HW = (G.RW + 1) >> 1, n_slots = HW * G.RH, half = (int)blockDim.x >> 1;
+    const int colour = (int)threadIdx.x >= half, slot = (int)threadIdx.x - colour * half;
+    const int row = slot / HW, y = G.ly0 + row;
+    const int odd = (G.lx0 + y + colour) & 1;  // the pixel's column in the region is odd
+    const int x = G.lx0 + 2 * (slot - row * HW) + odd;
+    const bool mine = row < G.RH && x < G.lx0 + G.RW;
+    const int X = K.g * x, Y = K.g * y, lw = K.lw, lh = K.lh, n_d = lw * lh;
+    uint32_t* const own = smem + colour * n_slots + slot;
+    const uint32_t* const other = smem + (colour ^ 1) * n_slots + slot;
+    const size_t g = (size_t)y * w + x;
+    const bool ok = mine && idx_ok(g_bounds, kBoundsTileRead, (long long)g, (long long)w * h) &&
+                    (!FF_DEBUG_BOUNDS || idx_ok(g_bounds, kBoundsTileSmem, 2 * n_slots - 1, dyn_smem_bytes() / 4));
+    uint32_t a[C::kSectors][8];
+    load_all<C>(K.fa, ok ? feat_index(X, Y, lw) : 0, n_d, kBoundsOwn, a);
+    uint32_t cur = !ok ? 0u : DF ? __ldcg(io.flow_in + g) : io.flow_in[g];
+    int c = !ok ? 0 : DF ? __ldcg(io.cost_in + g) : io.cost_in[g];
+    uint32_t left = cur, right = cur, up = cur, down = cur;  // the flow last tried from each side
+    if (ok) *own = cur;
+    __syncthreads();
+    int ahead = INT_MAX, ox = 0, oy = 0;  // the next random candidate: its cost around the present flow, its offset
+#pragma unroll 1
+    for (int it = 0; it < n_iter; it++) {
+        const uint32_t k2 = pixel_key(iter_key(P, io.t0 + it), X, Y);
+        const SweepRegions& S = s_regions[it & 1];
+        if (it + 1 < n_iter) s_regions[(it + 1) & 1].set(G, w, h, kHaloPerIter * (n_iter - 2 - it));
+#pragma unroll 1
+        for (int j = 0; j < 8; j++) {
+            const int d = j >> 1;
+            if ((j & 1) == colour) {
+                const int4 r = S.r[j];
+                if (ok && x >= r.x && x < r.z && y >= r.y && y < r.w) {
+                    const int dx = (d & 1) ? 1 : -1, dy = (d & 2) ? 1 : -1;
+                    // the horizontal neighbour has the pixel's slot, or the next one on its side
+                    const int s1 = odd == (d & 1) ? dx : 0, s2 = dy * HW;
+                    const bool v1 = (unsigned)(x + dx) < (unsigned)w && idx_ok(g_bounds, kBoundsSmemN1, slot + s1, n_slots);
+                    const bool v2 = (unsigned)(y + dy) < (unsigned)h && idx_ok(g_bounds, kBoundsSmemN2, slot + s2, n_slots);
+                    const uint32_t f1 = v1 ? other[s1] : cur, f2 = v2 ? other[s2] : cur;
+                    const uint32_t l1 = (d & 1) ? right : left, l2 = (d & 2) ? down : up;
+                    if (d & 1) right = f1; else left = f1;
+                    if (d & 2) down = f2; else up = f2;
+                    const uint32_t cur0 = cur;
+                    const bool e1 = f1 != l1 && f1 != cur && in_level(X + flow_x(f1), Y + flow_y(f1), lw, lh);
+                    const bool e2 = f2 != l2 && f2 != cur && f2 != f1 && in_level(X + flow_x(f2), Y + flow_y(f2), lw, lh);
+                    if (e1 || e2) {
+                        uint32_t b1[C::kSectors][8] = {}, b2[C::kSectors][8] = {};
+                        if (e1) load_all<C>(K.fb, feat_index(X + flow_x(f1), Y + flow_y(f1), lw), n_d, kBoundsCand1, b1);
+                        if (e2) load_all<C>(K.fb, feat_index(X + flow_x(f2), Y + flow_y(f2), lw), n_d, kBoundsCand2, b2);
+                        if (e1) {
+                            const int s = dist_all<C>(a, b1);
+                            if (s < c) { cur = f1; c = s; }
+                        }
+                        if (e2) {
+                            const int s = dist_all<C>(a, b2);
+                            if (s < c) { cur = f2; c = s; }
+                        }
+                    }
+                    if (d >= 1 && (ox != 0 || oy != 0)) {
+                        const int fx = flow_x(cur) + ox, fy = flow_y(cur) + oy;
+                        const int s = cur == cur0 ? ahead : score<C>(K, X, Y, a, fx, fy);
+                        if (s < c) { cur = pack_flow(fx, fy); c = s; }
+                    }
+                    if (cur != cur0) *own = cur;
+                }
+            } else if (j >= 1 && j < 7) {  // the pixel's next half-sweep is j + 1, with a random candidate
+                const int4 r = S.r[j + 1];
+                if (ok && x >= r.x && x < r.z && y >= r.y && y < r.w) {
+                    const int dn = (j + 1) >> 1;
+                    ox = K.offset(mix32(k2 ^ (uint32_t)(2 * dn)));
+                    oy = K.offset(mix32(k2 ^ (uint32_t)(2 * dn + 1)));
+                    ahead = score<C>(K, X, Y, a, flow_x(cur) + ox, flow_y(cur) + oy);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (!ok || x < G.x0 || x >= G.x1 || y < G.y0 || y >= G.y1) return;
+    if (!idx_ok(g_bounds, kBoundsTileWrite, (long long)g, (long long)w * h)) return;
+    io.flow_out[g] = cur;
+    io.cost_out[g] = c;
+}
+
 // One tile of one problem: load the tile and its halo, run n_iter iterations in shared memory, write the tile.
 // With DF, a dataflow task, the state was written by other CTAs of the running launch and is therefore read from L2.
-template <class C, bool DF>
+template <class C, bool DF, bool RES>
 __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int tile, const PropLaunch& L,
                                                       uint32_t* smem, const TileIO& io) {
     __shared__ SweepRegions s_regions[2];  // of iterations it and it + 1
@@ -353,6 +470,10 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
     int32_t* scost = reinterpret_cast<int32_t*>(smem + G.RW * G.RH);
     const SweepConst K = sweep_const(P, L.grid != 0);
     s_regions[0].set(G, w, h, kHaloPerIter * (n_iter - 1));
+    if constexpr (RES) {
+        propagate_tile_resident<C, DF>(K, G, P, smem, io, s_regions);
+        return;
+    }
 
     for (int i = threadIdx.x; i < G.RW * G.RH; i += blockDim.x) {
         int r = i / G.RW, c = i - r * G.RW;
@@ -599,6 +720,13 @@ bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow) {
     int pitch = 8;
     while (pitch < RW) pitch *= 2;
     return dataflow && pass_pixels >= kListedPixels && threads >= 256 && 4 * RW >= 3 * pitch;
+}
+
+// The resident variant takes every tile it can (regions of at most one pixel per thread): in the same tiles it is never
+// slower (8x8 pixels and 256 threads: 55 instead of 73 us at level 4 of the 1242x375 pair, 72 instead of 80 at level 3).
+bool prop_resident(int tw, int th, int n_iter, int threads) {
+    const int H = kHaloPerIter * n_iter;
+    return 2 * ((tw + 2 * H + 1) / 2) * (th + 2 * H) <= threads;
 }
 
 extern __shared__ __align__(16) uint32_t g_smem[];
@@ -865,7 +993,7 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
 // round trips, of which this leaves out two (level 4 of the 1242x375 pair 64 -> 61 us, level 3 79 -> 77; the three
 // launches of the 32x24 level of the 128x96 pair 61 -> 58).  queue[i] = (problem index, tile index in problem).
 // Instantiated for 128, 256 and 512 threads, per cost (direct variant).
-template <int THREADS, class C>
+template <int THREADS, class C, bool RES>
 __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
     PropLaunch L) {
@@ -878,7 +1006,7 @@ __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
         const int2 e = queue[q];
         const PropProblem& P = probs[e.x];
         const TileIO io = {P.flow_in, P.cost_in, P.flow_out, P.cost_out, P.t0, P.n_iter};
-        propagate_tile_direct<C, false>(P, e.y, L, g_smem, io);
+        propagate_tile_direct<C, false, RES>(P, e.y, L, g_smem, io);
         if (G >= n_tiles) return;
         if (threadIdx.x == 0) s_next = next;
         __syncthreads();
@@ -914,8 +1042,8 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <int THREADS, class C, bool LISTED>
-__global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_propagate_df(
+template <int THREADS, class C, Variant V>
+__global__ __launch_bounds__(THREADS, (V == kListed ? 1024 : 512) / THREADS) void k_propagate_df(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
     PropLaunch L, TileLayout LT) {
     grid_dependency_sync();
@@ -932,7 +1060,7 @@ __global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_pr
             const int ti = k / per_iter;
             q = ti * n_tiles + (int)blockIdx.x + (k - ti * per_iter) * G;
         } else {
-            if (!LISTED || k == 0) {
+            if (V != kListed || k == 0) {
                 if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
                 __syncthreads();
             }
@@ -947,7 +1075,7 @@ __global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_pr
         const TileIO io = {src_alt ? P.flow_alt : P.flow_in, src_alt ? P.cost_alt : P.cost_in,
                            t == T - 1 ? P.flow_out : dst_alt ? P.flow_alt : P.flow_in,
                            t == T - 1 ? P.cost_out : dst_alt ? P.cost_alt : P.cost_in, P.t0 + t, 1};
-        if constexpr (LISTED)
+        if constexpr (V == kListed)
             if (threadIdx.x == 32) tile_setup(P, e.y, L), tile_shared().io = io;
         bool ok = true;
         if (t > 0 && !failed && threadIdx.x < 9) {  // one waiting thread per tile of the 3x3 neighbourhood
@@ -964,10 +1092,10 @@ __global__ __launch_bounds__(THREADS, (LISTED ? 1024 : 512) / THREADS) void k_pr
             }
         }
         failed = __syncthreads_or(!ok) != 0 || failed;
-        if constexpr (LISTED)
+        if constexpr (V == kListed)
             propagate_tile_listed<C, THREADS>(P, LT, L.affine ? nullptr : counter, &s_next);
         else
-            propagate_tile_direct<C, true>(P, e.y, L, g_smem, io);
+            propagate_tile_direct<C, true, V == kResident>(P, e.y, L, g_smem, io);
         __syncthreads();  // every store of the tile is issued
         if (threadIdx.x == 64 && !L.withhold) {
             __threadfence();
@@ -1165,24 +1293,33 @@ using PropClusterKernel = void (*)(const PropProblem*, PropLaunch);
 
 using PropDataflowKernel = void (*)(const PropProblem*, const int2*, int, int*, PropLaunch, TileLayout);
 
-template <class C>
+template <class C, bool RES>
 PropKernel prop_kernel_t(int threads) {
-    return threads == 128 ? k_propagate<128, C> : threads == 512 ? k_propagate<512, C> : k_propagate<256, C>;
+    return threads == 128   ? k_propagate<128, C, RES>
+           : threads == 512 ? k_propagate<512, C, RES>
+                            : k_propagate<256, C, RES>;
 }
-PropKernel prop_kernel(int threads, int cost) {
-    return cost == FF_COST_CENSUS ? prop_kernel_t<CostCensus>(threads) : prop_kernel_t<CostSad>(threads);
+PropKernel prop_kernel(int threads, int cost, bool resident) {
+    if (resident)
+        return cost == FF_COST_CENSUS ? prop_kernel_t<CostCensus, true>(threads) : prop_kernel_t<CostSad, true>(threads);
+    return cost == FF_COST_CENSUS ? prop_kernel_t<CostCensus, false>(threads) : prop_kernel_t<CostSad, false>(threads);
 }
 
-// The direct variant is instantiated for 128, 256 and 512 threads, the listed one for 256 and 512 (prop_listed).
-template <class C>
-PropDataflowKernel prop_df_kernel_t(int threads, bool listed) {
-    if (listed) return threads == 512 ? k_propagate_df<512, C, true> : k_propagate_df<256, C, true>;
-    return threads == 128   ? k_propagate_df<128, C, false>
-           : threads == 512 ? k_propagate_df<512, C, false>
-                            : k_propagate_df<256, C, false>;
+// The listed variant is instantiated for 256 and 512 threads (prop_listed), the others for 128 too.
+template <class C, Variant V>
+PropDataflowKernel prop_df_kernel_t(int threads) {
+    if constexpr (V != kListed)
+        if (threads == 128) return k_propagate_df<128, C, V>;
+    return threads == 512 ? k_propagate_df<512, C, V> : k_propagate_df<256, C, V>;
 }
-PropDataflowKernel prop_df_kernel(int threads, int cost, bool listed) {
-    return cost == FF_COST_CENSUS ? prop_df_kernel_t<CostCensus>(threads, listed) : prop_df_kernel_t<CostSad>(threads, listed);
+template <Variant V>
+PropDataflowKernel prop_df_kernel_v(int threads, int cost) {
+    return cost == FF_COST_CENSUS ? prop_df_kernel_t<CostCensus, V>(threads) : prop_df_kernel_t<CostSad, V>(threads);
+}
+PropDataflowKernel prop_df_kernel(int threads, int cost, Variant v) {
+    return v == kListed     ? prop_df_kernel_v<kListed>(threads, cost)
+           : v == kResident ? prop_df_kernel_v<kResident>(threads, cost)
+                            : prop_df_kernel_v<kDirect>(threads, cost);
 }
 
 // The cluster form is instantiated for 256 and 512 threads, per cost.
@@ -1216,12 +1353,14 @@ cudaError_t init_kernel_attributes() {
     if (e0 != cudaSuccess) return e0;
     for (int cost : {FF_COST_WHT_SAD, FF_COST_CENSUS}) {
         for (int t : {128, 256, 512}) {
-            const void* ks[3] = {reinterpret_cast<const void*>(prop_kernel(t, cost)),
-                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, false)),
-                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, true))};
-            for (int v = 0; v < 3; v++) {
+            const void* ks[5] = {reinterpret_cast<const void*>(prop_kernel(t, cost, false)),
+                                 reinterpret_cast<const void*>(prop_kernel(t, cost, true)),
+                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, kDirect)),
+                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, kResident)),
+                                 reinterpret_cast<const void*>(prop_df_kernel(t, cost, kListed))};
+            for (int v = 0; v < 5; v++) {
                 cudaError_t e = cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)(v == 2 ? kMaxTileSmem : kMaxPropSmem));
+                                                     (int)(v == 4 ? kMaxTileSmem : kMaxPropSmem));
                 if (e != cudaSuccess) return e;
             }
         }
@@ -1238,14 +1377,20 @@ cudaError_t init_kernel_attributes() {
 bool prop_threads_ok(int threads) { return threads == 128 || threads == 256 || threads == 512; }
 
 int prop_blocks_per_sm(size_t smem, int threads, int cost, bool dataflow, bool listed) {
-    int n = 0;
-    const void* k = dataflow ? reinterpret_cast<const void*>(prop_df_kernel(threads, cost, listed))
-                             : reinterpret_cast<const void*>(prop_kernel(threads, cost));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
-    }
-    return n > 0 ? n : 1;
+    const auto blocks = [&](auto* k) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, reinterpret_cast<const void*>(k), threads, smem) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return 1;
+        }
+        return n > 0 ? n : 1;
+    };
+    if (listed) return blocks(prop_df_kernel(threads, cost, kListed));
+    // of whichever of the other two the launch takes (prop_resident)
+    if (dataflow)
+        return std::min(blocks(prop_df_kernel(threads, cost, kDirect)), blocks(prop_df_kernel(threads, cost, kResident)));
+    return std::min(blocks(prop_kernel(threads, cost, false)), blocks(prop_kernel(threads, cost, true)));
 }
 
 int prop_cluster_capacity(int cluster, int threads, int cost, size_t smem) {
@@ -1269,11 +1414,12 @@ void launch_propagate(const PropProblem* probs_dev, const int2* queue_dev, int n
         return;
     }
     const size_t smem = prop_launch_smem(L.tw, L.th, L.max_iter, L.listed != 0);
+    const bool resident = prop_resident(L.tw, L.th, L.dataflow > 0 ? 1 : L.max_iter, L.threads);
     if (L.dataflow > 0)
-        launch_k(prop_df_kernel(L.threads, L.cost, L.listed != 0), dim3(grid), dim3(L.threads), smem, st, probs_dev,
+        launch_k(prop_df_kernel(L.threads, L.cost, L.listed ? kListed : resident ? kResident : kDirect), dim3(grid), dim3(L.threads), smem, st, probs_dev,
                  queue_dev, n_tiles, counter_dev, L, tile_layout(L.tw, L.th));
     else
-        launch_k(prop_kernel(L.threads, L.cost), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles,
+        launch_k(prop_kernel(L.threads, L.cost, resident), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles,
                  counter_dev, L);
 }
 
