@@ -351,6 +351,17 @@ TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow
     return {16, 8, 1, 256, 0};
 }
 
+// What ff_match_pair_noalloc reckons its scratch with (a queue entry per tile, a problem per launch): which frames fit is
+// part of its interface and must not move with the rule above, whose small tiles and single iterations need some
+// kilobytes more at the coarse levels.
+TileCfg compact_cfg(const ff_ctx* c, int64_t level_pix_all, int T) {
+    const int64_t slots = (int64_t)c->n_sms * 2;
+    if (level_pix_all / (32 * 32) >= 2 * slots) return {32, 32, 1, 256, 0};
+    if (level_pix_all / (32 * 16) >= 2 * slots) return {32, 16, 1, 256, 0};
+    if (level_pix_all / (16 * 16) >= slots) return {16, 16, std::min(2, T), 256, 0};
+    return {8, 8, std::min(3, T), 256, 0};
+}
+
 ff_status enqueue_launch(ff_ctx* c, const Launch& L) {
     cudaStream_t st = c->stream;
     switch (L.kind) {
@@ -1258,10 +1269,10 @@ bool pyr_view(const ff_pyr* p, PyrView* out) {
 
 // The configuration for pass `level` (a level s or a sub-scale grid s + 8k) of size w x h, in the tile or (if
 // dataflow_ok) the dataflow form: the override if it is of one of these forms, else the best of them the
-// autotuner timed for this size with the nearest number of directions per launch, else the default.  A dataflow
-// configuration where it is not wanted becomes its tiles with one iteration per launch.
+// autotuner timed for this size with the nearest number of directions per launch, else the default (or the compact
+// one).  A dataflow configuration where it is not wanted becomes its tiles with one iteration per launch.
 TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs, int64_t level_pix_all,
-                            bool dataflow_ok) {
+                            bool dataflow_ok, bool compact) {
     const int T = c->prm.iters;
     TileCfg tc;
     if (level >= 0 && level < kMaxPasses && c->forced[level].threads > 0 && c->forced[level].cluster == 0) {
@@ -1279,7 +1290,7 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
                 best_d = d;
             }
         }
-        tc = best ? *best : default_cfg(c, level_pix_all, T, dataflow_ok);
+        tc = best ? *best : compact ? compact_cfg(c, level_pix_all, T) : default_cfg(c, level_pix_all, T, dataflow_ok);
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);

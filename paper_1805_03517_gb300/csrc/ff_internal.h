@@ -414,9 +414,10 @@ bool ctx_view(const ff_ctx* c, CtxView* out);
 bool ctx_owns_live_pyr(const ff_ctx* c, const ff_pyr* p);
 bool pyr_view(const ff_pyr* p, PyrView* out);
 // the launch configuration of a pass (level s, or its sub-scale grid s + 8k) of size w x h for the server and the
-// no-allocation entry point, which launch the tile form and (dataflow_ok) the dataflow form, never the cluster form
+// no-allocation entry point, which launch the tile form and (dataflow_ok) the dataflow form, never the cluster form; compact: an untuned
+// pass takes the configuration the no-allocation entry point's scratch is reckoned with instead of the fastest one
 TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs, int64_t level_pix_all,
-                            bool dataflow_ok);
+                            bool dataflow_ok, bool compact);
 // the context's error word of the bounded device waits, allocated on first use (null if that fails)
 int* ctx_err_word(ff_ctx* c);
 // cudaMalloc on behalf of a context; fails as out of memory while the context's FF_OPT_TEST_FAIL_ALLOCS count lasts

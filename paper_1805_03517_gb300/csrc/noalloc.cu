@@ -120,54 +120,65 @@ extern "C" ff_status ff_match_pair_noalloc(ff_ctx* c, const ff_pyr* a, const ff_
     sa.L = L;
     sa.T = T;
     TileChoice tc[kMaxLevels];
-    int grid[kMaxLevels];
     int total_launches = 0;
-    for (int s = L - 1; s >= 0; s--) {
-        tc[s] = ctx_level_choice(c, s, A.ws[s], A.hs[s], 1, (int64_t)A.ws[s] * A.hs[s], false);
-        sa.k[s] = tc[s].k;
-        sa.n_launch[s] = (T + tc[s].k - 1) / tc[s].k;
-        sa.first_launch[s] = total_launches;
-        total_launches += sa.n_launch[s];
-        int tiles_x = (A.ws[s] + tc[s].tw - 1) / tc[s].tw;
-        sa.ntiles[s] = tiles_x * ((A.hs[s] + tc[s].th - 1) / tc[s].th);
+    int* counters = nullptr;
+    int32_t* dist = nullptr;
+    // carves the scratch array and returns the bytes it takes
+    const auto carve = [&](bool compact) {
+        total_launches = 0;
+        for (int s = L - 1; s >= 0; s--) {
+            tc[s] = ctx_level_choice(c, s, A.ws[s], A.hs[s], 1, (int64_t)A.ws[s] * A.hs[s], false, compact);
+            sa.k[s] = tc[s].k;
+            sa.n_launch[s] = (T + tc[s].k - 1) / tc[s].k;
+            sa.first_launch[s] = total_launches;
+            total_launches += sa.n_launch[s];
+            int tiles_x = (A.ws[s] + tc[s].tw - 1) / tc[s].tw;
+            sa.ntiles[s] = tiles_x * ((A.hs[s] + tc[s].th - 1) / tc[s].th);
+            PropProblem& p = sa.base[s];
+            p.fa = cost_desc(A, s, cv.cost);
+            p.fb = cost_desc(B, s, cv.cost);
+            p.w = A.ws[s];
+            p.h = A.hs[s];
+            p.tiles_x = tiles_x;
+            p.level = s;
+            p.dir = dir;
+            p.seed = cv.seed;
+            p.rs_radius = (uint16_t)cv.rs_radius;
+            p.T = (uint16_t)T;
+        }
+        sa.total_launches = total_launches;
+
+        size_t off = 0;
+        auto take = [&](size_t bytes) {
+            size_t o = off;
+            off += align256(bytes);
+            return static_cast<char*>(base) + o;
+        };
+        sa.seed_dst = reinterpret_cast<SeedProblem*>(take(sizeof(SeedProblem)));
+        sa.ho_dst = reinterpret_cast<HandoverProblem*>(take(sizeof(HandoverProblem) * L));
+        sa.props = reinterpret_cast<PropProblem*>(take(sizeof(PropProblem) * total_launches));
+        counters = reinterpret_cast<int*>(take(sizeof(int) * total_launches));
+        for (int s = 0; s < L; s++) sa.queue[s] = reinterpret_cast<int2*>(take(sizeof(int2) * sa.ntiles[s]));
+        dist = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * A.n_coarse));
+        for (int s = 0; s < L; s++) {
+            size_t n = (size_t)A.ws[s] * A.hs[s];
+            for (int k = 0; k < 2; k++) {
+                sa.flow[s][k] = reinterpret_cast<uint32_t*>(take(n * 4));
+                sa.cost[s][k] = reinterpret_cast<int32_t*>(take(n * 4));
+            }
+        }
+        return off;
+    };
+    // reject what does not fit; the configurations for speed, unless only the compact ones fit
+    constexpr size_t kBytes = (size_t)FF_NOALLOC_SCRATCH_BYTES;
+    if (carve(true) > kBytes)
+        return err(FF_ERR_ARG, "pyramids too large for the fixed scratch of ff_match_pair_noalloc");
+    if (carve(false) > kBytes) carve(true);
+    int grid[kMaxLevels];
+    for (int s = 0; s < L; s++) {
         size_t smem = prop_smem_bytes(tc[s].tw, tc[s].th, tc[s].k);
         grid[s] = std::min(sa.ntiles[s], prop_blocks_per_sm(smem, tc[s].threads, cv.cost, false, false) * cv.n_sms);
-        PropProblem& p = sa.base[s];
-        p.fa = cost_desc(A, s, cv.cost);
-        p.fb = cost_desc(B, s, cv.cost);
-        p.w = A.ws[s];
-        p.h = A.hs[s];
-        p.tiles_x = tiles_x;
-        p.level = s;
-        p.dir = dir;
-        p.seed = cv.seed;
-        p.rs_radius = (uint16_t)cv.rs_radius;
-        p.T = (uint16_t)T;
     }
-    sa.total_launches = total_launches;
-
-    // carve the scratch array; reject what does not fit
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        size_t o = off;
-        off += align256(bytes);
-        return static_cast<char*>(base) + o;
-    };
-    sa.seed_dst = reinterpret_cast<SeedProblem*>(take(sizeof(SeedProblem)));
-    sa.ho_dst = reinterpret_cast<HandoverProblem*>(take(sizeof(HandoverProblem) * L));
-    sa.props = reinterpret_cast<PropProblem*>(take(sizeof(PropProblem) * total_launches));
-    int* counters = reinterpret_cast<int*>(take(sizeof(int) * total_launches));
-    for (int s = 0; s < L; s++) sa.queue[s] = reinterpret_cast<int2*>(take(sizeof(int2) * sa.ntiles[s]));
-    int32_t* dist = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * A.n_coarse));
-    for (int s = 0; s < L; s++) {
-        size_t n = (size_t)A.ws[s] * A.hs[s];
-        for (int k = 0; k < 2; k++) {
-            sa.flow[s][k] = reinterpret_cast<uint32_t*>(take(n * 4));
-            sa.cost[s][k] = reinterpret_cast<int32_t*>(take(n * 4));
-        }
-    }
-    if (off > (size_t)FF_NOALLOC_SCRATCH_BYTES)
-        return err(FF_ERR_ARG, "pyramids too large for the fixed scratch of ff_match_pair_noalloc");
 
     SeedProblem& sp = sa.seed;
     sp.A = A.seed_desc;

@@ -253,7 +253,7 @@ ff_status admit(ff_server* s) {
             for (int g = 0; g <= grids_of(l, q.L, s->cv.sub_scales); g++) {  // tuning entries: pass l + 8g
                 const int gw = grid_dim(q.A.ws[l], g), gh = grid_dim(q.A.hs[l], g);
                 q.cfg[l][g] =
-                    ctx_level_choice(s->ctx, l + kMaxLevels * g, gw, gh, n_dirs, (int64_t)n_dirs * gw * gh, true);
+                    ctx_level_choice(s->ctx, l + kMaxLevels * g, gw, gh, n_dirs, (int64_t)n_dirs * gw * gh, true, false);
                 const TileChoice& t = q.cfg[l][g];
                 if (t.k < 1 || t.tw < 1 || t.th < 1 || !prop_threads_ok(t.threads) ||
                     prop_smem_bytes(t.tw, t.th, t.dataflow ? 1 : t.k) > kMaxPropSmem ||
