@@ -1291,6 +1291,11 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
             }
         }
         tc = best ? *best : compact ? compact_cfg(c, level_pix_all, T) : default_cfg(c, level_pix_all, T, dataflow_ok);
+        // A request of the server advances by a launch of the tile form per tick when many are in flight, so single
+        // iterations would hold it for as many ticks: such a pass runs as one launch of the dataflow form (16 mixed pairs
+        // served together 10.15 ms instead of 10.95; alone, a pass takes 72 to 79 us instead of 66 to 72).
+        if (!best && !compact && dataflow_ok && tc.dataflow == 0 && tc.k == 1)
+            tc = TileCfg{16, 12, 1, 512, 0, 0, 1};
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);
