@@ -15,9 +15,10 @@
 // upstream sides of each later half-sweep.  Recomputed halo pixels use exactly the inputs of the CTA that owns
 // them, so every tile's output equals the global schedule bit for bit.
 //
-// The work of a tile has two variants.  The direct one gives every pixel of a half-sweep a thread, which scores the
-// pixel's candidates.  The listed one skips the candidates that are known not to be cheaper and gives threads only to
-// the pixels left (see there); dataflow launches of enough pixels to keep the GPU busy take it (prop_listed).
+// The work of a tile has three variants.  The direct one gives every pixel of a half-sweep a thread, which scores the
+// pixel's candidates.  The resident one gives every pixel of the region its own thread for the whole launch; tiles small
+// enough take it (prop_resident).  The listed one skips the candidates that are known not to be cheaper and gives threads
+// only to the pixels left; dataflow launches of enough pixels to keep the GPU busy take it (prop_listed).
 #include <climits>
 #include <cstddef>
 
@@ -448,7 +449,8 @@ __device__ __forceinline__ void propagate_tile_resident(const SweepConst& K, con
     io.cost_out[g] = c;
 }
 
-// One tile of one problem: load the tile and its halo, run n_iter iterations in shared memory, write the tile.
+// One tile of one problem: load the tile and its halo, run n_iter iterations in shared memory (RES: with the resident
+// variant), write the tile.
 // With DF, a dataflow task, the state was written by other CTAs of the running launch and is therefore read from L2.
 template <class C, bool DF, bool RES>
 __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int tile, const PropLaunch& L,
@@ -723,7 +725,7 @@ bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow) {
 }
 
 // The resident variant takes every tile it can (regions of at most one pixel per thread): in the same tiles it is never
-// slower (8x8 pixels and 256 threads: 55 instead of 73 us at level 4 of the 1242x375 pair, 72 instead of 80 at level 3).
+// slower (8x8 pixels and 256 threads: 57 instead of 73 us at level 4 of the 1242x375 pair, 72 instead of 80 at level 3).
 bool prop_resident(int tw, int th, int n_iter, int threads) {
     const int H = kHaloPerIter * n_iter;
     return 2 * ((tw + 2 * H + 1) / 2) * (th + 2 * H) <= threads;
@@ -992,7 +994,7 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
 // before is worked on, and a launch with a CTA per tile takes none.  At small levels a launch is a chain of memory
 // round trips, of which this leaves out two (level 4 of the 1242x375 pair 64 -> 61 us, level 3 79 -> 77; the three
 // launches of the 32x24 level of the 128x96 pair 61 -> 58).  queue[i] = (problem index, tile index in problem).
-// Instantiated for 128, 256 and 512 threads, per cost (direct variant).
+// Instantiated for 128, 256 and 512 threads, per cost, direct and resident.
 template <int THREADS, class C, bool RES>
 __global__ __launch_bounds__(THREADS, 512 / THREADS) void k_propagate(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
