@@ -190,6 +190,25 @@ void prop_fit_tile(int& tw, int& th);
 // the listed variant of the dataflow form.
 bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow);
 
+// Listed variant: whom the change of a pixel's flow in half-sweep stamp - 1 of an iteration still concerns when the next
+// one starts: bit 0 the pixel right of it (whose left neighbour it is), 1 left, 2 below, 3 above.  A pixel of colour k
+// last tried its left neighbour in half-sweep 4 + k, its right and lower ones in 6 + k, its upper one in 2 + k.  Stamp 0:
+// no half-sweep changed it.  Larger stamps than 8 are in no state word a task writes, but what a task reads after a wait
+// that expired is whatever the buffer holds: they concern nobody.
+constexpr uint32_t still_concerned_table() {  // one nibble per stamp 1..8
+    uint32_t m = 0;
+    for (int s = 1; s <= 8; s++) {
+        const int j = s - 1, k = 1 - (j & 1);  // the neighbours have the other colour
+        const uint32_t n = (j > 4 + k ? 1u : 0u) | (j > 6 + k ? 2u : 0u) | (j > 2 + k ? 4u : 0u) | (j > 6 + k ? 8u : 0u);
+        m |= n << (4 * (s - 1));
+    }
+    return m;
+}
+__host__ __device__ constexpr uint32_t still_concerned(uint32_t stamp) {
+    constexpr uint32_t table = still_concerned_table();
+    return stamp - 1u < 8u ? table >> (4 * (stamp - 1u)) & 15u : 0u;
+}
+
 // Cluster form of a propagation launch: the n CTAs of a cluster split a w x h problem into bx x by blocks
 // (bx * by = n), CTA r owning block (r % bx, r / bx) with columns [i*w/bx, (i+1)*w/bx) and rows
 // [j*h/by, (j+1)*h/by).  The divisor pair with the smallest total block perimeter (w*by + h*bx) is taken, among

@@ -534,22 +534,10 @@ __device__ __forceinline__ uint32_t todo_bits(int d) {  // those of direction d
 //   bits 13..11  the random candidates of the next iteration that have to be scored (screen)
 //   bits 3..0    1 + the half-sweep of the iteration that last changed the flow, 0: none did
 // In shared memory the flags are in the todo bytes.
+// (Other words than these are read here after a wait that expired; every use of their bits stays in range.)
 constexpr int kCostShift = 14, kFlagShift = 11;
 constexpr uint32_t kStampMask = 15u, kCostMax = (1u << (32 - kCostShift)) - 1;
 __device__ __forceinline__ uint32_t pack_state(int cost) { return min((uint32_t)cost, kCostMax) << kCostShift; }
-// Whom the change of a pixel's flow in half-sweep stamp - 1 still concerns when the next iteration starts: bit 0 the
-// pixel right of it (whose left neighbour it is), 1 left, 2 below, 3 above.  A pixel of colour k last tried its left
-// neighbour in half-sweep 4 + k, its right and lower ones in 6 + k, its upper one in 2 + k; one nibble per stamp.
-constexpr uint32_t still_concerned() {
-    uint32_t m = 0;
-    for (int s = 1; s <= 8; s++) {
-        const int j = s - 1, k = 1 - (j & 1);  // the neighbours have the other colour
-        const uint32_t n = (j > 4 + k ? 1u : 0u) | (j > 6 + k ? 2u : 0u) | (j > 2 + k ? 4u : 0u) | (j > 6 + k ? 8u : 0u);
-        m |= n << (4 * (s - 1));
-    }
-    return m;
-}
-
 // Constants of a problem, in shared memory.
 struct alignas(16) Sweep {
     const void* fa;
@@ -936,7 +924,7 @@ __device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, cons
             g_smem[T.o_state() + sidx] = first ? pack_state((int)st) : st >> kCostShift << kCostShift;
             if (!first && (st & ((1u << kCostShift) - 1))) {
                 const uint32_t live = st >> kFlagShift & 7u, stamp = st & kStampMask;
-                const uint32_t who = stamp ? still_concerned() >> (4 * (stamp - 1)) & 15u : 0u;
+                const uint32_t who = still_concerned(stamp);
                 const int colour = (S.lx0 + c + S.ly0 + r) & 1, b = ((r + 1) << T.slots) + (c >> 1);
                 if (live) atomicOr(todo + colour * T.todo_words() + (b >> 2), live << (8 * (b & 3) + 4));
                 if (who) mark_neighbours(todo + (colour ^ 1) * T.todo_words(), b, T.slots, c, who);
