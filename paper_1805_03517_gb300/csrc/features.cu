@@ -162,7 +162,7 @@ __device__ __forceinline__ void st_sector(void* p, const uint32_t (&v)[8]) {
                  : "memory");
 }
 
-// acc + the sum of the four bytes of a, weighted by the signed bytes of b.
+// The sum of the four bytes of a, weighted by the signed bytes of b.
 __device__ __forceinline__ int dp4a_us(uint32_t a, uint32_t b) {
     int d;
     asm("dp4a.u32.s32 %0, %1, %2, 0;" : "=r"(d) : "r"(a), "r"(b));
@@ -323,12 +323,11 @@ __device__ __forceinline__ void wht_tile(const WhtLevel& L, int t, uint8_t (&win
 #pragma unroll
             for (int rr = 0; rr < N; rr++) {
                 if (y0 + rr >= L.h) break;
-                constexpr int kBias = (int)0x80008000u;  // offset binary in both halves
-                const int px = P[rr].x + kBias, py = P[rr].y + kBias, dx = D[rr].x + kBias, dy = D[rr].y + kBias;
-                const int2 q = P[rr + 4], t = D[rr + 4];
-                const uint32_t out[8] = {(uint32_t)(px + q.x), (uint32_t)(py + q.y), (uint32_t)(px - q.x),
-                                         (uint32_t)(py - q.y), (uint32_t)(dx - t.x), (uint32_t)(dy - t.y),
-                                         (uint32_t)(dx + t.x), (uint32_t)(dy + t.y)};
+                const uint32_t px = offset_pair(P[rr].x), py = offset_pair(P[rr].y), dx = offset_pair(D[rr].x),
+                               dy = offset_pair(D[rr].y);
+                const uint32_t qx = (uint32_t)P[rr + 4].x, qy = (uint32_t)P[rr + 4].y, tx = (uint32_t)D[rr + 4].x,
+                               ty = (uint32_t)D[rr + 4].y;
+                const uint32_t out[8] = {px + qx, py + qy, px - qx, py - qy, dx - tx, dy - ty, dx + tx, dy + ty};
                 if (idx_ok(g_bounds, kBoundsFeat, feat_index(x, y0 + rr, L.w), (long long)L.w * L.h))
                     st_sector(dst + rr * row, out);
             }

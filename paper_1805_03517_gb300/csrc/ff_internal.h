@@ -309,6 +309,10 @@ __host__ __device__ __forceinline__ int feature_coef(int16_t stored) {
     return (int)(int16_t)((uint16_t)stored ^ 0x8000u);
 }
 
+// Two packed sums lo + 65536 * hi, in offset binary in both halves.  The halves' bias does not fit a signed integer
+// together with a negative upper sum.
+__host__ __device__ __forceinline__ uint32_t offset_pair(int packed) { return (uint32_t)packed + 0x80008000u; }
+
 // Position of pixel (x, y) in a colour-split feature map of width w.
 __host__ __device__ __forceinline__ int feat_index(int x, int y, int w) {
     return y * w + ((x & 1) ? ((w + 1) >> 1) + (x >> 1) : (x >> 1));
