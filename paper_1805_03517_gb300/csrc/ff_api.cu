@@ -679,8 +679,8 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
         if (df) tc.k = T;  // one launch, one iteration per tile task
         const bool listed = !cl && prop_listed(level_pix, tc.tw, tc.threads, df);
         if (listed) prop_fit_tile(tc.tw, tc.th);
-        const size_t smem = cl ? 0 : prop_launch_smem(tc.tw, tc.th, df ? 1 : tc.k, listed);
-        const int blocks = cl ? 0 : prop_blocks_per_sm(smem, tc.threads, cost, df, listed) * c->n_sms;
+        const int blocks =
+            cl ? 0 : prop_blocks_per_sm(tc.tw, tc.th, df ? 1 : tc.k, tc.threads, cost, df, listed) * c->n_sms;
         for (int t0 = 0; t0 < T; t0 += tc.k) {
             int n_iter = std::min(tc.k, T - t0);
             bool last = t0 + n_iter == T;
@@ -1101,7 +1101,7 @@ void wave_shape(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k, 
     for (const DirJob& j : jobs)
         n += (int64_t)((grid_dim(j.a->ws[s], k) + t.tw - 1) / t.tw) * ((grid_dim(j.a->hs[s], k) + t.th - 1) / t.th);
     *tiles = n;
-    *slots = (int64_t)prop_blocks_per_sm(prop_smem_bytes(t.tw, t.th, t.k), t.threads, c->prm.cost, false, false) * c->n_sms;
+    *slots = (int64_t)prop_blocks_per_sm(t.tw, t.th, t.k, t.threads, c->prm.cost, false, false) * c->n_sms;
 }
 
 // A launch whose last wave is a small remainder of tiles runs at about the speed of one more full wave.  The

@@ -243,8 +243,8 @@ cudaError_t seed_load_kernel();        // loads k_seed onto the current device (
 // fixed scratch array) and the kernels it launches, and returns the array's device address.
 cudaError_t noalloc_prepare(void** scratch);
 bool prop_threads_ok(int threads);
-// resident CTAs per SM of the tile form (dataflow: of its dataflow kernel)
-int prop_blocks_per_sm(size_t smem, int threads, int cost, bool dataflow, bool listed);
+// Resident CTAs per SM of a tile or dataflow launch, in the variant it takes (n_iter: iterations per tile task).
+int prop_blocks_per_sm(int tw, int th, int n_iter, int threads, int cost, bool dataflow, bool listed);
 // Tile form (L.cluster == 0): queue_dev[i] = (problem index, tile index); counter_dev must be zero when the launch
 // starts; `grid` CTAs.  Dataflow form (L.dataflow = T): the same queue, taken T times (iteration-major).  Cluster form: problem i is probs_dev[i], `grid` = number of problems x L.cluster CTAs;
 // queue_dev and counter_dev are unused.

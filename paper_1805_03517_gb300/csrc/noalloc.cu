@@ -176,8 +176,8 @@ extern "C" ff_status ff_match_pair_noalloc(ff_ctx* c, const ff_pyr* a, const ff_
     if (carve(false) > kBytes) carve(true);
     int grid[kMaxLevels];
     for (int s = 0; s < L; s++) {
-        size_t smem = prop_smem_bytes(tc[s].tw, tc[s].th, tc[s].k);
-        grid[s] = std::min(sa.ntiles[s], prop_blocks_per_sm(smem, tc[s].threads, cv.cost, false, false) * cv.n_sms);
+        grid[s] = std::min(sa.ntiles[s], cv.n_sms * prop_blocks_per_sm(tc[s].tw, tc[s].th, tc[s].k, tc[s].threads,
+                                                                       cv.cost, false, false));
     }
 
     SeedProblem& sp = sa.seed;

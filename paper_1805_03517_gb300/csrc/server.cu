@@ -478,12 +478,11 @@ ff_status tick(ff_server* s) {
             }
             pi++;
         }
-        const size_t smem = prop_launch_smem(k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.listed != 0);
         const int nq = (int)(qi - q0);
         PropLaunch pl{k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.threads, s->cv.cost, k.grid};
         pl.listed = k.listed;
-        const int slots =
-            prop_blocks_per_sm(smem, k.threads, s->cv.cost, k.dataflow != 0, k.listed != 0) * s->cv.n_sms;
+        const int slots = s->cv.n_sms * prop_blocks_per_sm(k.tw, k.th, k.dataflow ? 1 : k.n_iter, k.threads, s->cv.cost,
+                                                           k.dataflow != 0, k.listed != 0);
         if (k.dataflow) {
             pl.dataflow = k.n_iter;
             pl.affine = k.dataflow == 2;
