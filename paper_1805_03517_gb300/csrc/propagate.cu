@@ -978,12 +978,15 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
 }
 
 // Persistent launch: each CTA takes tiles from the launch's queue until it is empty, so the last wave has no idle tail.
-// CTA b starts with entry b; the others are taken with an atomic counter (zeroed before the launch) while the tile
-// before is worked on, and a launch with a CTA per tile takes none.  At small levels a launch is a chain of memory
-// round trips, of which this leaves out two (level 4 of the 1242x375 pair 64 -> 61 us, level 3 79 -> 77; the three
-// launches of the 32x24 level of the 128x96 pair 61 -> 58).  queue[i] = (problem index, tile index in problem).
+// CTA b starts with entry b; the others are taken with an atomic counter (zeroed before the launch), and a launch with a
+// CTA per tile takes none.  At small levels a launch is a chain of memory round trips, of which this leaves out two (level
+// 4 of the 1242x375 pair 64 -> 61 us, level 3 79 -> 77; the three launches of the 32x24 level of the 128x96 pair 61 -> 58).
+// A CTA takes its next tile when it has finished the one before: taken at that one's start, the launch's last tiles are
+// held by CTAs that are still busy while others idle (a 128x96 pair in 8x8 tiles of three iterations 298 instead of 268
+// us, a 1242x375 direction without allocation 1001 instead of 953, 1920x1080 in 32x32 tiles under Census 2985, 2960).
+// queue[i] = (problem index, tile index in problem).
 // Instantiated for 128, 256 and 512 threads, per cost, direct and resident.
-// The direct Census kernel is held to the registers of three CTAs of 256 threads per SM (79; unbounded it takes 96, two
+// The direct Census kernel is held to the registers of three CTAs of 256 threads per SM (78; unbounded it takes 92, two
 // CTAs): a 1920x1080 pair in 32x32 tiles 2.98 instead of 3.63 ms, a 1024x436 direction without allocation 524 instead of
 // 630 us.
 template <int THREADS, class C, bool RES>
@@ -994,14 +997,12 @@ __global__ __launch_bounds__(THREADS, (RES || C::kSectors > 1 ? 512 : 768) / THR
     __shared__ int s_next;
     const int G = (int)gridDim.x;
     for (int q = (int)blockIdx.x; q < n_tiles; q = s_next) {
-        int next = n_tiles;
-        if (G < n_tiles && threadIdx.x == 0) next = G + atomicAdd(counter, 1);
         const int2 e = queue[q];
         const PropProblem& P = probs[e.x];
         const TileIO io = {P.flow_in, P.cost_in, P.flow_out, P.cost_out, P.t0, P.n_iter};
         propagate_tile_direct<C, false, RES>(P, e.y, L, g_smem, io);
         if (G >= n_tiles) return;
-        if (threadIdx.x == 0) s_next = next;
+        if (threadIdx.x == 0) s_next = G + atomicAdd(counter, 1);
         __syncthreads();
     }
 }
