@@ -138,12 +138,6 @@ struct FineWht {
     int tiles = 0;                  // CTAs
 };
 
-struct TileCfg {
-    int tw, th, k, threads, spec;  // tile interior, iterations fused per launch, CTA size (spec: without effect)
-    int cluster = 0;               // > 0: the cluster form with this many CTAs per problem (tw, th unused)
-    int dataflow = 0;              // 1: the dataflow form (every iteration in one launch; k unused), 2: affine
-};
-
 // Candidate propagation configurations (tile shape, fused iterations, CTA size) the autotuner times per level.
 const TileCfg kCands[] = {
     {64, 32, 1, 256, 0}, {32, 32, 1, 256, 0}, {32, 16, 1, 256, 0}, {16, 16, 1, 256, 0}, {32, 16, 2, 256, 0},
@@ -312,6 +306,8 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
     return true;
 }
 
+}  // namespace
+
 // Default propagation configuration of a pass that has not been tuned, by its pixels (all problems of its launches):
 // from 28,000 pixels the queue variant of the dataflow form (every iteration in one launch, no resident grid needed),
 // in tiles small enough to keep every SM busy; below, where a pass is a chain of half-sweeps on a few SMs, the tile
@@ -319,19 +315,27 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
 // a CTA, and below 4,000 pixels with two iterations per launch, whose halo idle SMs absorb.  The lines are the near-best
 // of a sweep over single pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both
 // costs.  Passes the listed variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the
-// largest that leave the queue more tiles than the 608 CTAs an SM's 2048 threads make (a Census distance is a third of
-// the work, so larger tiles still balance).  Levels 0 to 4 of the 1242x375 pair (us): 531, 221, 109, 72 and 50 instead of
-// 844, 375, 294, 113 and 75 with the rule before these variants; of the 1920x1080 pair 1674, 527, 240, 113 and 67
-// instead of 3280, 935, 594, 475 and 142.
-TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow_ok) {
+// largest that leave the queue more tiles than the 608 CTAs of four per SM (a Census distance is a third of the work, so
+// larger tiles still balance).
+// In one or two iterations there is little to skip and few launches to save.  There a Census pass takes the tile form,
+// whose direct kernel has three CTAs per SM and the dataflow form's two, and a WHT-SAD pass of one iteration from 300,000
+// pixels too (two iterations, 893 k pixels, us: WHT-SAD 276 in 32x32 dataflow tiles, 285 in 32x32 tiles of the tile form,
+// 383 listed in 24x16; Census 147, 123 and 211; 112 k pixels, Census: 31 in 16x16 tiles of the tile form, 45 in 20x12
+// dataflow tiles).
+// Levels 0 to 4 of the 1242x375 pair (us): 531, 221, 109, 72 and 50 instead of 844, 375, 294, 113 and 75 with the rule
+// before these variants; of the 1920x1080 pair 1674, 527, 240, 113 and 67 instead of 3280, 935, 594, 475 and 142.
+TileCfg ff::default_cfg(int n_sms, int cost, int64_t level_pix_all, int T, bool dataflow_ok) {
+    const bool census = cost == FF_COST_CENSUS;
+    if (census ? T == 1 || (T == 2 && level_pix_all <= 130000) : T == 1 && level_pix_all >= 300000) dataflow_ok = false;
     if (dataflow_ok) {
-        if (prop_listed(level_pix_all, 56, 256, true)) {
-            const int64_t tiles = c->prm.cost == FF_COST_CENSUS ? 650 : 1000;
+        if (prop_listed(level_pix_all, 56, 256, T, true)) {
+            const int64_t tiles = census ? 650 : 1000;
             if (level_pix_all >= tiles * 56 * 40) return {56, 40, 1, 256, 0, 0, 1};
             if (level_pix_all >= tiles * 56 * 24) return {56, 24, 1, 256, 0, 0, 1};
             if (level_pix_all >= tiles * 56 * 16) return {56, 16, 1, 256, 0, 0, 1};
             return {24, 16, 1, 256, 0, 0, 1};
         }
+        if (level_pix_all >= 300000) return {32, 32, 1, 256, 0, 0, census ? 0 : 1};  // two iterations
         if (level_pix_all > 200000) return {24, 24, 1, 256, 0, 0, 1};
         if (level_pix_all > 130000) return {24, 16, 1, 256, 0, 0, 1};
         if (level_pix_all > 75000) return {20, 12, 1, 256, 0, 0, 1};
@@ -341,15 +345,17 @@ TileCfg default_cfg(const ff_ctx* c, int64_t level_pix_all, int T, bool dataflow
     }
     if (level_pix_all <= 4000) return {8, 4, std::min(2, T), 512, 0};
     if (level_pix_all <= 20000) return {8, 8, 1, 256, 0};
-    if (level_pix_all <= 28000) return {16, 12, 1, 512, 0};
+    if (level_pix_all <= 28000 && !(census && T <= 2)) return {16, 12, 1, 512, 0};
     // tile form only (a launch per group of iterations): large tiles with one iteration per launch when the level
     // fills the GPU, otherwise small tiles with fused iterations
-    const int64_t slots = (int64_t)c->n_sms * 2;
+    const int64_t slots = (int64_t)n_sms * 2;
     if (level_pix_all / (32 * 32) >= 2 * slots) return {32, 32, 1, 256, 0};
     if (level_pix_all / (32 * 16) >= 2 * slots) return {32, 16, 1, 256, 0};
     if (level_pix_all > 50000) return {16, 16, 1, 256, 0};
     return {16, 8, 1, 256, 0};
 }
+
+namespace {
 
 // What ff_match_pair_noalloc reckons its scratch with (a queue entry per tile, a problem per launch): which frames fit is
 // part of its interface and must not move with the rule above, whose small tiles and single iterations need some
@@ -671,13 +677,14 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
             tc.k = std::min(tc.k, T);
         } else {
             auto it = c->tuned.find(TuneKey{pass, gdim(jobs[0].a->ws[s], k), gdim(jobs[0].a->hs[s], k), nj, T});
-            tc = it != c->tuned.end() ? it->second : default_cfg(c, level_pix, T, true);
+            tc = it != c->tuned.end() ? it->second : default_cfg(c->n_sms, cost, level_pix, T, true);
         }
         size_t cl_smem = 0;
-        if (tc.cluster > 0 && !cluster_fits(c, jobs, s, k, tc, &cl_smem)) tc = default_cfg(c, level_pix, T, true);
+        if (tc.cluster > 0 && !cluster_fits(c, jobs, s, k, tc, &cl_smem))
+            tc = default_cfg(c->n_sms, cost, level_pix, T, true);
         const bool cl = tc.cluster > 0, df = tc.dataflow > 0;
         if (df) tc.k = T;  // one launch, one iteration per tile task
-        const bool listed = !cl && prop_listed(level_pix, tc.tw, tc.threads, df);
+        const bool listed = !cl && prop_listed(level_pix, tc.tw, tc.threads, T, df);
         if (listed) prop_fit_tile(tc.tw, tc.th);
         const int blocks =
             cl ? 0 : prop_blocks_per_sm(tc.tw, tc.th, df ? 1 : tc.k, tc.threads, cost, df, listed) * c->n_sms;
@@ -1290,16 +1297,18 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
                 best_d = d;
             }
         }
-        tc = best ? *best : compact ? compact_cfg(c, level_pix_all, T) : default_cfg(c, level_pix_all, T, dataflow_ok);
+        tc = best      ? *best
+             : compact ? compact_cfg(c, level_pix_all, T)
+                       : default_cfg(c->n_sms, c->prm.cost, level_pix_all, T, dataflow_ok);
         // A request of the server advances by a launch of the tile form per tick when many are in flight, so single
         // iterations would hold it for as many ticks: such a pass runs as one launch of the dataflow form (16 mixed pairs
         // served together 10.15 ms instead of 10.95; alone, a pass takes 72 to 79 us instead of 66 to 72).
-        if (!best && !compact && dataflow_ok && tc.dataflow == 0 && tc.k == 1)
+        if (!best && !compact && dataflow_ok && tc.dataflow == 0 && tc.k == 1 && T > 1 && level_pix_all <= 28000)
             tc = TileCfg{16, 12, 1, 512, 0, 0, 1};
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);
-    const bool listed = prop_listed(level_pix_all, tc.tw, tc.threads, tc.dataflow > 0);
+    const bool listed = prop_listed(level_pix_all, tc.tw, tc.threads, T, tc.dataflow > 0);
     if (listed) prop_fit_tile(tc.tw, tc.th);
     return {tc.tw, tc.th, tc.k, tc.threads, listed, tc.dataflow};
 }

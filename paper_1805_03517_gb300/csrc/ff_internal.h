@@ -186,9 +186,9 @@ size_t prop_launch_smem(int tw, int th, int n_iter, bool listed);  // dynamic sh
 // The largest tiles prop_smem_bytes allows are shrunk to what a launch of the listed variant can take (results do not
 // depend on the tiles).
 void prop_fit_tile(int& tw, int& th);
-// Whether a pass of that many pixels (all problems of its launch), in tiles tw wide on CTAs of that many threads, takes
-// the listed variant of the dataflow form.
-bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow);
+// Whether a pass of that many pixels (all problems of its launch) and T iterations, in tiles tw wide on CTAs of that many
+// threads, takes the listed variant of the dataflow form.
+bool prop_listed(int64_t pass_pixels, int tw, int threads, int T, bool dataflow);
 
 // Listed variant: whom the change of a pixel's flow in half-sweep stamp - 1 of an iteration still concerns when the next
 // one starts: bit 0 the pixel right of it (whose left neighbour it is), 1 left, 2 below, 3 above.  A pixel of colour k
@@ -208,6 +208,17 @@ __host__ __device__ constexpr uint32_t still_concerned(uint32_t stamp) {
     constexpr uint32_t table = still_concerned_table();
     return stamp - 1u < 8u ? table >> (4 * (stamp - 1u)) & 15u : 0u;
 }
+
+// Launch configuration of a pass.
+struct TileCfg {
+    int tw, th, k, threads, spec;  // tile interior, iterations fused per launch, CTA size (spec: without effect, kept
+                                   // for ff_get_tuning)
+    int cluster = 0;               // > 0: the cluster form with this many CTAs per problem (tw, th unused)
+    int dataflow = 0;              // 1: the dataflow form (every iteration in one launch; k unused), 2: affine
+};
+// That of an untuned pass of level_pix_all pixels (all problems of its launches) and T iterations, in the tile and (if
+// dataflow_ok) the dataflow form.
+TileCfg default_cfg(int n_sms, int cost, int64_t level_pix_all, int T, bool dataflow_ok);
 
 // Cluster form of a propagation launch: the n CTAs of a cluster split a w x h problem into bx x by blocks
 // (bx * by = n), CTA r owning block (r % bx, r / bx) with columns [i*w/bx, (i+1)*w/bx) and rows

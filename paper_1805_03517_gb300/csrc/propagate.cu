@@ -704,12 +704,13 @@ void prop_fit_tile(int& tw, int& th) {
 // 640x480 direction 795 us listed, 639 direct: a launch per iteration leaves the screening's tail exposed), 128 threads
 // (level 0 of the 1242x375 pair in 48x24 tiles: 900 us listed, 663 direct), and regions that leave over a quarter of
 // their power-of-two rows empty (64x32 tiles, 72 wide: 688, 669 direct).
-constexpr int64_t kListedPixels = 300000;
-bool prop_listed(int64_t pass_pixels, int tw, int threads, bool dataflow) {
+// In the first iteration nothing is known yet, so a pass of one iteration has only the lists' cost (level 0 of the 1920x1080
+// pair 764 us, 612 direct), and one of two gains from larger passes on (893 k pixels 301, 276 direct; 1.26 M 213, 272).
+bool prop_listed(int64_t pass_pixels, int tw, int threads, int T, bool dataflow) {
     const int RW = tw + 2 * kHaloPerIter;
     int pitch = 8;
     while (pitch < RW) pitch *= 2;
-    return dataflow && pass_pixels >= kListedPixels && threads >= 256 && 4 * RW >= 3 * pitch;
+    return dataflow && T >= 2 && pass_pixels >= (T == 2 ? 1200000 : 300000) && threads >= 256 && 4 * RW >= 3 * pitch;
 }
 
 // The resident variant takes every tile it can (regions of at most one pixel per thread): in the same tiles it is never

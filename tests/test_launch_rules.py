@@ -1,0 +1,62 @@
+"""The host rules that choose an untuned pass's variant and launch configuration (prop_listed, default_cfg), called on the
+CPU from the library's own objects.  In the first iteration of a pass the listed variant has nothing to skip, so it
+takes no pass of one iteration and one of two only from larger sizes on; every configuration of the default rule is one
+that ff_set_tuning accepts."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1805_03517_gb300 import build as B
+
+PROGRAM = r"""
+#include <cstdio>
+#include "ff_internal.h"
+using namespace ff;
+int main() {
+    for (int cost : {FF_COST_WHT_SAD, FF_COST_CENSUS})
+        for (int T : {1, 2, 3, 6, 255})
+            for (int df = 0; df < 2; df++)
+                for (long long px = 1; px < (1ll << 33); px += 1 + px / 64) {
+                    const TileCfg c = default_cfg(152, cost, px, T, df != 0);
+                    const bool listed = prop_listed(px, c.tw, c.threads, T, c.dataflow > 0);
+                    std::printf("%d %d %d %lld %d %d %d %d %d %d %d %d\n", cost, T, df, px, c.tw, c.th, c.k, c.threads,
+                                c.cluster, c.dataflow, (int)listed,
+                                (int)(prop_threads_ok(c.threads) && prop_smem_bytes(c.tw, c.th, c.k) <= kMaxPropSmem));
+                }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rows(tmp_path_factory):
+    B.build()
+    d = tmp_path_factory.mktemp("rules")
+    src, exe = d / "rules.cu", d / "rules"
+    src.write_text(PROGRAM)
+    objs = [os.path.join(B.BUILD, s.replace(".cu", ".o")) for s in B.SOURCES]
+    r = subprocess.run([B.nvcc(), *B.ARCH, *B.FLAGS, "-o", str(exe), str(src), *objs], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
+    return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
+
+
+def test_default_configurations_are_valid(rows):
+    for cost, T, df, px, tw, th, k, threads, cluster, dataflow, listed, fits in rows:
+        assert fits and 1 <= k <= T and cluster == 0 and dataflow in (0, 1), (cost, T, df, px)
+        assert not dataflow or (df and k == 1 and tw >= 4 and th >= 4), (cost, T, df, px)
+        assert not listed or dataflow, (cost, T, df, px)
+
+
+def test_listed_variant_by_iterations(rows):
+    for cost, T, df, px, *_, dataflow, listed, _ in rows:
+        least = {1: None, 2: 1_200_000}.get(T, 300_000)
+        assert listed == int(bool(df) and least is not None and px >= least), (cost, T, df, px)
+
+
+def test_few_census_iterations_take_the_tile_form(rows):
+    """Its direct kernel has three CTAs per SM under the Census cost, the dataflow form's has two."""
+    for cost, T, df, px, *_, dataflow, listed, _ in rows:
+        if cost == 1 and (T == 1 or (T == 2 and not listed and (px <= 130_000 or px >= 300_000))):
+            assert not dataflow, (T, df, px)
