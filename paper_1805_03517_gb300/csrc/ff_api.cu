@@ -290,6 +290,8 @@ bool cfg_fits(const TileCfg& t) {
     return t.cluster > 0 || prop_smem_bytes(t.tw, t.th, t.dataflow ? 1 : t.k) <= kMaxPropSmem;
 }
 
+int64_t tiles_of(int w, int h, const TileCfg& t) { return (int64_t)((w + t.tw - 1) / t.tw) * ((h + t.th - 1) / t.th); }
+
 // Whether the cluster form of `t` can run pass (s, k) of these jobs: a partition of every problem, its shared
 // memory within the limit, and clusters of that shape launchable on this device.  *smem: the largest CTA's bytes.
 bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k, const TileCfg& t, size_t* smem) {
@@ -328,7 +330,7 @@ TileCfg ff::default_cfg(int n_sms, int cost, int64_t level_pix_all, int T, bool 
     const bool census = cost == FF_COST_CENSUS;
     if (census ? T == 1 || (T == 2 && level_pix_all <= 130000) : T == 1 && level_pix_all >= 300000) dataflow_ok = false;
     if (dataflow_ok) {
-        if (prop_listed(level_pix_all, 56, 256, T, true)) {
+        if (level_pix_all >= prop_listed_pixels(T)) {
             const int64_t tiles = census ? 650 : 1000;
             if (level_pix_all >= tiles * 56 * 40) return {56, 40, 1, 256, 0, 0, 1};
             if (level_pix_all >= tiles * 56 * 24) return {56, 24, 1, 256, 0, 0, 1};
@@ -684,7 +686,10 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
             tc = default_cfg(c->n_sms, cost, level_pix, T, true);
         const bool cl = tc.cluster > 0, df = tc.dataflow > 0;
         if (df) tc.k = T;  // one launch, one iteration per tile task
-        const bool listed = !cl && prop_listed(level_pix, tc.tw, tc.threads, T, df);
+        int64_t tiles = 0;
+        for (int j = 0; j < nj && !cl; j++)
+            tiles += tiles_of(gdim(jobs[j].a->ws[s], k), gdim(jobs[j].a->hs[s], k), tc);
+        const bool listed = !cl && prop_listed(level_pix, tiles, tc.tw, tc.threads, T, df, c->n_sms);
         if (listed) prop_fit_tile(tc.tw, tc.th);
         const int blocks =
             cl ? 0 : prop_blocks_per_sm(tc.tw, tc.th, df ? 1 : tc.k, tc.threads, cost, df, listed) * c->n_sms;
@@ -1105,8 +1110,7 @@ ff_status run_jobs(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vector
 void wave_shape(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k, const TileCfg& t, int64_t* tiles,
                 int64_t* slots) {
     int64_t n = 0;
-    for (const DirJob& j : jobs)
-        n += (int64_t)((grid_dim(j.a->ws[s], k) + t.tw - 1) / t.tw) * ((grid_dim(j.a->hs[s], k) + t.th - 1) / t.th);
+    for (const DirJob& j : jobs) n += tiles_of(grid_dim(j.a->ws[s], k), grid_dim(j.a->hs[s], k), t);
     *tiles = n;
     *slots = (int64_t)prop_blocks_per_sm(t.tw, t.th, t.k, t.threads, c->prm.cost, false, false) * c->n_sms;
 }
@@ -1308,7 +1312,8 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);
-    const bool listed = prop_listed(level_pix_all, tc.tw, tc.threads, T, tc.dataflow > 0);
+    const bool listed = prop_listed(level_pix_all, n_dirs * tiles_of(w, h, tc), tc.tw, tc.threads, T, tc.dataflow > 0,
+                                    c->n_sms);
     if (listed) prop_fit_tile(tc.tw, tc.th);
     return {tc.tw, tc.th, tc.k, tc.threads, listed, tc.dataflow};
 }

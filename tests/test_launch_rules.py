@@ -19,7 +19,8 @@ int main() {
             for (int df = 0; df < 2; df++)
                 for (long long px = 1; px < (1ll << 33); px += 1 + px / 64) {
                     const TileCfg c = default_cfg(152, cost, px, T, df != 0);
-                    const bool listed = prop_listed(px, c.tw, c.threads, T, c.dataflow > 0);
+                    const long long tiles = px / (c.tw * c.th) + 1;  // at least: of frames that are whole tiles
+                    const bool listed = prop_listed(px, tiles, c.tw, c.threads, T, c.dataflow > 0, 152);
                     std::printf("%d %d %d %lld %d %d %d %d %d %d %d %d\n", cost, T, df, px, c.tw, c.th, c.k, c.threads,
                                 c.cluster, c.dataflow, (int)listed,
                                 (int)(prop_threads_ok(c.threads) && prop_smem_bytes(c.tw, c.th, c.k) <= kMaxPropSmem));
@@ -29,17 +30,21 @@ int main() {
 """
 
 
-@pytest.fixture(scope="module")
-def rows(tmp_path_factory):
+def run(program, d):
+    """The lines of numbers a main() linked with the library's objects prints."""
     B.build()
-    d = tmp_path_factory.mktemp("rules")
     src, exe = d / "rules.cu", d / "rules"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     objs = [os.path.join(B.BUILD, s.replace(".cu", ".o")) for s in B.SOURCES]
     r = subprocess.run([B.nvcc(), *B.ARCH, *B.FLAGS, "-o", str(exe), str(src), *objs], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
     out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
     return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
+
+
+@pytest.fixture(scope="module")
+def rows(tmp_path_factory):
+    return run(PROGRAM, tmp_path_factory.mktemp("rules"))
 
 
 def test_default_configurations_are_valid(rows):
@@ -60,3 +65,17 @@ def test_few_census_iterations_take_the_tile_form(rows):
     for cost, T, df, px, *_, dataflow, listed, _ in rows:
         if cost == 1 and (T == 1 or (T == 2 and not listed and (px <= 130_000 or px >= 300_000))):
             assert not dataflow, (T, df, px)
+
+
+# pixels, tiles, tile width, threads, iterations -> listed
+CASES = [((465_750, 198, 56, 256, 3), 0), ((465_750, 198, 56, 256, 6), 0), ((465_750, 198, 56, 256, 10), 1),
+         ((465_750, 607, 24, 256, 9), 0), ((465_750, 608, 24, 256, 3), 1), ((465_750, 303, 24, 512, 6), 0),
+         ((465_750, 304, 24, 512, 6), 1), ((2_073_600, 720, 120, 256, 5), 0), ((2_073_600, 720, 120, 256, 6), 1),
+         ((2_073_600, 2000, 64, 256, 6), 0), ((2_073_600, 2000, 56, 128, 6), 0), ((299_999, 2000, 24, 256, 6), 0)]
+
+
+def test_listed_variant_by_tiles(tmp_path):
+    """It has twice the direct variant's CTAs, which fewer tiles leave idle, unless enough iterations are skipped."""
+    calls = "".join("    std::printf(\"%%d\\n\", (int)prop_listed(%d, %d, %d, %d, %d, true, 152));\n" % c for c, _ in CASES)
+    got = run('#include <cstdio>\n#include "ff_internal.h"\nusing namespace ff;\nint main() {\n' + calls + "}\n", tmp_path)
+    assert [g[0] for g in got] == [want for _, want in CASES]
