@@ -318,7 +318,9 @@ bool cluster_fits(const ff_ctx* c, const std::vector<DirJob>& jobs, int s, int k
 // of a sweep over single pairs of 128x96 to 1920x1080, one and two directions, and six 1242x375 pairs, under both
 // costs.  Passes the listed variant takes (prop_listed) have tiles whose regions (tile + 8) are a power of two wide, the
 // largest that leave the queue more tiles than the 608 CTAs of four per SM (a Census distance is a third of the work, so
-// larger tiles still balance).
+// larger tiles still balance).  Below, the lines are where such tiles had left passes slower than before the listed variant
+// (893 k pixels, WHT-SAD, three iterations: 56x16 373 us, 24x24 414, 24x16 498, before 439; 446 k, Census, six iterations:
+// 24x24 205, 24x16 260, before 252).
 // In one or two iterations there is little to skip and few launches to save.  There a Census pass takes the tile form,
 // whose direct kernel has three CTAs per SM and the dataflow form's two, and a WHT-SAD pass of one iteration from 300,000
 // pixels too (two iterations, 893 k pixels, us: WHT-SAD 276 in 32x32 dataflow tiles, 285 in 32x32 tiles of the tile form,
@@ -334,7 +336,8 @@ TileCfg ff::default_cfg(int n_sms, int cost, int64_t level_pix_all, int T, bool 
             const int64_t tiles = census ? 650 : 1000;
             if (level_pix_all >= tiles * 56 * 40) return {56, 40, 1, 256, 0, 0, 1};
             if (level_pix_all >= tiles * 56 * 24) return {56, 24, 1, 256, 0, 0, 1};
-            if (level_pix_all >= tiles * 56 * 16) return {56, 16, 1, 256, 0, 0, 1};
+            if (level_pix_all >= (census ? tiles * 56 * 16 : 850000)) return {56, 16, 1, 256, 0, 0, 1};
+            if (level_pix_all >= (census ? 400000 : 600000)) return {24, 24, 1, 256, 0, 0, 1};
             return {24, 16, 1, 256, 0, 0, 1};
         }
         if (level_pix_all >= 300000) return {32, 32, 1, 256, 0, 0, census ? 0 : 1};  // two iterations

@@ -67,6 +67,15 @@ def test_few_census_iterations_take_the_tile_form(rows):
             assert not dataflow, (T, df, px)
 
 
+@pytest.mark.parametrize("cost,T,px,tile", [(0, 3, 892_928, (56, 16)), (0, 6, 892_928, (56, 16)), (0, 3, 700_000, (24, 24)),
+                                            (1, 3, 446_464, (24, 24)), (1, 6, 465_750, (24, 24)), (0, 6, 320_000, (24, 16)),
+                                            (1, 6, 320_000, (24, 16)), (1, 6, 620_000, (56, 16))])
+def test_listed_tiles(rows, cost, T, px, tile):
+    """Passes of a size at which 24x16 tiles were measured slower than the former rule take larger ones."""
+    near = min((r for r in rows if r[0] == cost and r[1] == T and r[2]), key=lambda r: abs(r[3] - px))
+    assert (near[4], near[5]) == tile and near[10], near
+
+
 # pixels, tiles, tile width, threads, iterations -> listed
 CASES = [((465_750, 198, 56, 256, 3), 0), ((465_750, 198, 56, 256, 6), 0), ((465_750, 198, 56, 256, 10), 1),
          ((465_750, 607, 24, 256, 9), 0), ((465_750, 608, 24, 256, 3), 1), ((465_750, 303, 24, 512, 6), 0),
