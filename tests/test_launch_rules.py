@@ -88,3 +88,32 @@ def test_listed_variant_by_tiles(tmp_path):
     calls = "".join("    std::printf(\"%%d\\n\", (int)prop_listed(%d, %d, %d, %d, %d, true, 152));\n" % c for c, _ in CASES)
     got = run('#include <cstdio>\n#include "ff_internal.h"\nusing namespace ff;\nint main() {\n' + calls + "}\n", tmp_path)
     assert [g[0] for g in got] == [want for _, want in CASES]
+
+
+FIT = r"""
+#include <cstdio>
+#include "ff_internal.h"
+using namespace ff;
+int main() {
+    long long n = 0, shrunk = 0, bad = 0;
+    for (int tw = 4; tw <= 1024; tw++)
+        for (int th = 4; th <= 1024; th++) {
+            if (prop_smem_bytes(tw, th, 1) > kMaxPropSmem) continue;  // ff_set_tuning refuses it
+            int w = tw, h = th, slots = 4;
+            prop_fit_tile(w, h);
+            while (2 * slots < w + 2 * kHaloPerIter) slots *= 2;
+            n++;
+            shrunk += w != tw || h != th;
+            bad += w > tw || h > th || w < 4 || h < 4 || prop_launch_smem(w, h, 1, true) > kMaxTileSmem ||
+                   slots * (h + 2 * kHaloPerIter + 2) > 8192;  // a list entry has 13 bits for the slot
+        }
+    std::printf("%lld %lld %lld\n", n, shrunk, bad);
+    return 0;
+}
+"""
+
+
+def test_every_tile_fits_the_listed_variant(tmp_path):
+    n, shrunk, bad = run(FIT, tmp_path)[0]
+    accepted = sum(8 * (tw + 8) * (th + 8) <= 200 * 1024 for tw in range(4, 1025) for th in range(4, 1025))
+    assert n == accepted and 0 < shrunk < n and bad == 0
