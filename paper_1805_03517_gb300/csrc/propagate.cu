@@ -993,11 +993,12 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
 // us, a 1242x375 direction without allocation 1001 instead of 953, 1920x1080 in 32x32 tiles under Census 2985, 2960).
 // queue[i] = (problem index, tile index in problem).
 // Instantiated for 128, 256 and 512 threads, per cost, direct and resident.
-// The direct Census kernel is held to the registers of three CTAs of 256 threads per SM (78; unbounded it takes 92, two
-// CTAs): a 1920x1080 pair in 32x32 tiles 2.98 instead of 3.63 ms, a 1024x436 direction without allocation 524 instead of
-// 630 us.
+// The Census kernels are held to the registers of three CTAs of 256 threads per SM (direct 78, resident 71; unbounded 92
+// and 85, two CTAs).  Direct: a 1920x1080 pair in 32x32 tiles 2.98 instead of 3.63 ms, a 1024x436 direction without
+// allocation 524 instead of 630 us.  Resident: 27.9 k pixels in 8x8 tiles (448 of them, on 304 CTAs two rounds) 57 us
+// instead of 90.
 template <int THREADS, class C, bool RES>
-__global__ __launch_bounds__(THREADS, (RES || C::kSectors > 1 ? 512 : 768) / THREADS) void k_propagate(
+__global__ __launch_bounds__(THREADS, (C::kSectors > 1 ? 512 : 768) / THREADS) void k_propagate(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
     PropLaunch L) {
     grid_dependency_sync();
