@@ -1044,8 +1044,11 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// CTAs per SM: the listed variant is held to the registers of 1024 threads, the others to those of 512, under Census of
+// 640, so that five CTAs of 128 threads reside (direct 86 registers, unbounded 102 and four CTAs: level 0 of a 1920x1080
+// pair in 32x32 tiles 1628 instead of 1919 us).
 template <int THREADS, class C, Variant V>
-__global__ __launch_bounds__(THREADS, (V == kListed ? 1024 : 512) / THREADS) void k_propagate_df(
+__global__ __launch_bounds__(THREADS, (V == kListed ? 1024 : C::kSectors > 1 ? 512 : 640) / THREADS) void k_propagate_df(
     const PropProblem* __restrict__ probs, const int2* __restrict__ queue, int n_tiles, int* __restrict__ counter,
     PropLaunch L, TileLayout LT) {
     grid_dependency_sync();
