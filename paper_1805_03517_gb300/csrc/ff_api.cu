@@ -332,7 +332,7 @@ TileCfg ff::default_cfg(int n_sms, int cost, int64_t level_pix_all, int T, bool 
     const bool census = cost == FF_COST_CENSUS;
     if (census ? T == 1 || (T == 2 && level_pix_all <= 130000) : T == 1 && level_pix_all >= 300000) dataflow_ok = false;
     if (dataflow_ok) {
-        if (level_pix_all >= prop_listed_pixels(T)) {
+        if (level_pix_all >= prop_listed_pixels(T, cost)) {
             const int64_t tiles = census ? 650 : 1000;
             if (level_pix_all >= tiles * 56 * 40) return {56, 40, 1, 256, 0, 0, 1};
             if (level_pix_all >= tiles * 56 * 24) return {56, 24, 1, 256, 0, 0, 1};
@@ -692,7 +692,7 @@ ff_status build_plan(ff_ctx* c, const std::vector<DirJob>& jobs, const std::vect
         int64_t tiles = 0;
         for (int j = 0; j < nj && !cl; j++)
             tiles += tiles_of(gdim(jobs[j].a->ws[s], k), gdim(jobs[j].a->hs[s], k), tc);
-        const bool listed = !cl && prop_listed(level_pix, tiles, tc.tw, tc.threads, T, df, c->n_sms);
+        const bool listed = !cl && prop_listed(level_pix, tiles, tc.tw, tc.threads, T, cost, df, c->n_sms);
         if (listed) prop_fit_tile(tc.tw, tc.th);
         const int blocks =
             cl ? 0 : prop_blocks_per_sm(tc.tw, tc.th, df ? 1 : tc.k, tc.threads, cost, df, listed) * c->n_sms;
@@ -1315,8 +1315,8 @@ TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs
     }
     if (tc.dataflow > 0 && !dataflow_ok) tc = TileCfg{tc.tw, tc.th, 1, tc.threads, 0};
     tc.k = tc.dataflow > 0 ? T : std::min(tc.k, T);
-    const bool listed = prop_listed(level_pix_all, n_dirs * tiles_of(w, h, tc), tc.tw, tc.threads, T, tc.dataflow > 0,
-                                    c->n_sms);
+    const bool listed = prop_listed(level_pix_all, n_dirs * tiles_of(w, h, tc), tc.tw, tc.threads, T, c->prm.cost,
+                                    tc.dataflow > 0, c->n_sms);
     if (listed) prop_fit_tile(tc.tw, tc.th);
     return {tc.tw, tc.th, tc.k, tc.threads, listed, tc.dataflow};
 }

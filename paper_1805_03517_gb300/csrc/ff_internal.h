@@ -188,8 +188,8 @@ size_t prop_launch_smem(int tw, int th, int n_iter, bool listed);  // dynamic sh
 void prop_fit_tile(int& tw, int& th);
 // Whether a pass of that many pixels and tiles (all problems of its launch) and T iterations, in tiles tw wide on CTAs of
 // that many threads, takes the listed variant of the dataflow form; and the pixels from which one may.
-bool prop_listed(int64_t pass_pixels, int64_t pass_tiles, int tw, int threads, int T, bool dataflow, int n_sms);
-int64_t prop_listed_pixels(int T);
+bool prop_listed(int64_t pass_pixels, int64_t pass_tiles, int tw, int threads, int T, int cost, bool dataflow, int n_sms);
+int64_t prop_listed_pixels(int T, int cost);
 
 // Listed variant: whom the change of a pixel's flow in half-sweep stamp - 1 of an iteration still concerns when the next
 // one starts: bit 0 the pixel right of it (whose left neighbour it is), 1 left, 2 below, 3 above.  A pixel of colour k

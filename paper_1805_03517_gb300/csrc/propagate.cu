@@ -705,17 +705,21 @@ void prop_fit_tile(int& tw, int& th) {
 // (level 0 of the 1242x375 pair in 48x24 tiles: 900 us listed, 663 direct), and regions that leave over a quarter of
 // their power-of-two rows empty (64x32 tiles, 72 wide: 688, 669 direct).
 // In the first iteration nothing is known yet, so a pass of one iteration has only the lists' cost (level 0 of the 1920x1080
-// pair 764 us, 612 direct), and one of two gains from larger passes on (893 k pixels 301, 276 direct; 1.26 M 213, 272).
+// pair 764 us, 612 direct).  One of two gains from 1.2 M pixels on under Census (4.1 M 541 us, 594 direct in its best
+// tiles); under WHT-SAD it depends on the frames (1.26 M, shifted textures, 213, 272 direct; 2.07 M, an animation, 672,
+// 629), so it stays direct.
 // With fewer tiles than its CTAs (1024 threads per SM) a part of them idles, which the direct variant's half as many do
 // not, until enough iterations are skipped (466 k pixels in 198 tiles of 56x40, us, listed / direct: 434 / 274 with three
 // iterations, 716 / 539 with six, even with twelve).  Rows of 128 slots gain from more iterations on (1920x1080 direction
 // in 120x24 tiles 1164 / 925 with three).
-int64_t prop_listed_pixels(int T) { return T == 1 ? INT64_MAX : T == 2 ? 1200000 : 300000; }
-bool prop_listed(int64_t pass_pixels, int64_t pass_tiles, int tw, int threads, int T, bool dataflow, int n_sms) {
+int64_t prop_listed_pixels(int T, int cost) {
+    return T >= 3 ? 300000 : T == 2 && cost == FF_COST_CENSUS ? 1200000 : INT64_MAX;
+}
+bool prop_listed(int64_t pass_pixels, int64_t pass_tiles, int tw, int threads, int T, int cost, bool dataflow, int n_sms) {
     const int RW = tw + 2 * kHaloPerIter;
     int pitch = 8;
     while (pitch < RW) pitch *= 2;
-    return dataflow && pass_pixels >= prop_listed_pixels(T) && threads >= 256 && 4 * RW >= 3 * pitch &&
+    return dataflow && pass_pixels >= prop_listed_pixels(T, cost) && threads >= 256 && 4 * RW >= 3 * pitch &&
            (T >= 10 || pass_tiles * threads >= (int64_t)n_sms * 1024) && (T >= 6 || pitch <= 64);
 }
 

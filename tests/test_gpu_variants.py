@@ -1,7 +1,7 @@
 """Which variant of the propagation a pass takes, seen in a trace of the kernels, and that its results are the oracle's.
 The listed variant: batches of ragged frames with ten iterations (any number of tiles) in every tile shape, tiles that
 have to be shrunk to what it can hold (one by its bytes, two by its slots), both costs and the extreme search radii;
-passes just below and above its sizes with three and two iterations.  The debug-bounds build runs the shrunk tiles too."""
+passes just below and above its sizes with one to three iterations.  The debug-bounds build runs the shrunk tiles too."""
 import os
 import subprocess
 import sys
@@ -49,11 +49,19 @@ def test_listed_batch(ffm, tmp_path, cost, R):  # noqa: F811
 
 
 @pytest.mark.parametrize("n,h,w,T,last", [(1, 374, 401, 3, DIRECT), (1, 375, 401, 3, LISTED), (1, 375, 401, 2, DIRECT),
-                                          (1, 375, 401, 1, "k_propagate<"), (4, 374, 401, 2, DIRECT),
-                                          (4, 375, 401, 2, LISTED)])
+                                          (1, 375, 401, 1, "k_propagate<"), (4, 375, 401, 2, DIRECT)])
 def test_line_between_the_variants(ffm, tmp_path, n, h, w, T, last):  # noqa: F811
     """Passes of 299,948 and 300,750 pixels, and of four times as many."""
-    prm = configs.MatchParams(n_scales=4, iters=T, eps=1)
+    check_line(ffm, tmp_path, n, h, w, configs.MatchParams(n_scales=4, iters=T, eps=1), last)
+
+
+@pytest.mark.parametrize("n,h,w,T,last", [(1, 374, 401, 3, DIRECT), (1, 375, 401, 3, LISTED), (1, 375, 401, 2, "k_propagate<"),
+                                          (4, 374, 401, 2, "k_propagate<"), (4, 375, 401, 2, LISTED)])
+def test_line_between_the_variants_census(ffm, tmp_path, n, h, w, T, last):  # noqa: F811
+    check_line(ffm, tmp_path, n, h, w, configs.MatchParams(n_scales=4, iters=T, eps=1, cost=1), last)
+
+
+def check_line(ffm, tmp_path, n, h, w, prm, last):  # noqa: F811
     pairs = []
     for i in range(n):
         a = P.smooth_texture(800 + i, h, w)

@@ -20,7 +20,7 @@ int main() {
                 for (long long px = 1; px < (1ll << 33); px += 1 + px / 64) {
                     const TileCfg c = default_cfg(152, cost, px, T, df != 0);
                     const long long tiles = px / (c.tw * c.th) + 1;  // at least: of frames that are whole tiles
-                    const bool listed = prop_listed(px, tiles, c.tw, c.threads, T, c.dataflow > 0, 152);
+                    const bool listed = prop_listed(px, tiles, c.tw, c.threads, T, cost, c.dataflow > 0, 152);
                     std::printf("%d %d %d %lld %d %d %d %d %d %d %d %d\n", cost, T, df, px, c.tw, c.th, c.k, c.threads,
                                 c.cluster, c.dataflow, (int)listed,
                                 (int)(prop_threads_ok(c.threads) && prop_smem_bytes(c.tw, c.th, c.k) <= kMaxPropSmem));
@@ -56,7 +56,7 @@ def test_default_configurations_are_valid(rows):
 
 def test_listed_variant_by_iterations(rows):
     for cost, T, df, px, *_, dataflow, listed, _ in rows:
-        least = {1: None, 2: 1_200_000}.get(T, 300_000)
+        least = {1: None, 2: 1_200_000 if cost else None}.get(T, 300_000)
         assert listed == int(bool(df) and least is not None and px >= least), (cost, T, df, px)
 
 
@@ -80,12 +80,13 @@ def test_listed_tiles(rows, cost, T, px, tile):
 CASES = [((465_750, 198, 56, 256, 3), 0), ((465_750, 198, 56, 256, 6), 0), ((465_750, 198, 56, 256, 10), 1),
          ((465_750, 607, 24, 256, 9), 0), ((465_750, 608, 24, 256, 3), 1), ((465_750, 303, 24, 512, 6), 0),
          ((465_750, 304, 24, 512, 6), 1), ((2_073_600, 720, 120, 256, 5), 0), ((2_073_600, 720, 120, 256, 6), 1),
-         ((2_073_600, 2000, 64, 256, 6), 0), ((2_073_600, 2000, 56, 128, 6), 0), ((299_999, 2000, 24, 256, 6), 0)]
+         ((2_073_600, 2000, 64, 256, 6), 0), ((2_073_600, 2000, 56, 128, 6), 0), ((299_999, 2000, 24, 256, 6), 0),
+         ((2_073_600, 1575, 56, 256, 2), 0)]
 
 
 def test_listed_variant_by_tiles(tmp_path):
     """It has twice the direct variant's CTAs, which fewer tiles leave idle, unless enough iterations are skipped."""
-    calls = "".join("    std::printf(\"%%d\\n\", (int)prop_listed(%d, %d, %d, %d, %d, true, 152));\n" % c for c, _ in CASES)
+    calls = "".join("    std::printf(\"%%d\\n\", (int)prop_listed(%d, %d, %d, %d, %d, 0, true, 152));\n" % c for c, _ in CASES)
     got = run('#include <cstdio>\n#include "ff_internal.h"\nusing namespace ff;\nint main() {\n' + calls + "}\n", tmp_path)
     assert [g[0] for g in got] == [want for _, want in CASES]
 
