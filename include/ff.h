@@ -194,9 +194,9 @@ FF_API ff_status ff_match_frames(ff_ctx* ctx, int n_frames, const ff_frame* fram
 FF_API ff_status ff_autotune(ff_ctx* ctx, int n, const ff_pair_job* jobs, int reps);
 
 /* Propagation launch configuration of one level: tile interior (pixels), iterations fused per launch, threads
- * per CTA (128, 256 or 512).  speculate (0 or 1) has no effect: no kernel fetches the random candidate ahead of the
- * neighbour candidates any more.  With cluster = dataflow = 0 this is the tile form, one launch per iters_per_launch
- * iterations.
+ * per CTA (128, 256 or 512).  speculate (0 or 1) has no effect: it used to fetch the random candidate together with the
+ * neighbour candidates, which the variant of the kernels a launch takes now decides.  With cluster = dataflow = 0 this is
+ * the tile form, one launch per iters_per_launch iterations.
  * dataflow = 1 (cluster 0, iters_per_launch 1, speculate 0, tiles at least 4x4): every iteration of the level in
  * one persistent launch of one-iteration tile tasks, a tile starting iteration t as soon as the 3x3 tiles around
  * it have finished t - 1 (no launch boundary, hence no idle tail, between iterations); dataflow = 2 is its affine
@@ -365,9 +365,10 @@ FF_API ff_status ff_match_pair_noalloc(ff_ctx* ctx, const ff_pyr* a, const ff_py
  *   FF_OPT_WAIT_LIMIT            polls (1..2^30, default 2^22, about a second) before a device-side wait gives
  *                                up; the kernel then records the failure, cleans up and returns, and the next
  *                                ff_sync reports FF_ERR_TIMEOUT with the context still usable.
- *   FF_OPT_TEST_WITHHOLD_COPIES  1: the tensor-core seed issues no copies and the cluster form of the propagation
- *                                sends no block edges, so their waits can only expire (a test of the bounded
- *                                waits); 0 (default) normal operation.
+ *   FF_OPT_TEST_WITHHOLD_COPIES  1: the tensor-core seed issues no copies, the cluster form of the propagation sends no
+ *                                block edges and its dataflow form (which untuned passes take too) publishes no tile
+ *                                progress, so their waits can only expire (a test of the bounded waits); 0 (default)
+ *                                normal operation.
  *   FF_OPT_TEST_FAIL_ALLOCS      n >= 0: the next n device allocations made for this context (pyramids, plans, the
  *                                server's scratch and tables) fail as on an exhausted device, without calling the
  *                                allocator, so the calls that need them return FF_ERR_OOM and launch nothing (a test

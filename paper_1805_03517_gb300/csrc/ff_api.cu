@@ -145,7 +145,8 @@ const TileCfg kCands[] = {
     {32, 16, 1, 128, 0}, {16, 16, 1, 128, 0}, {16, 8, 2, 128, 0},  {8, 8, 3, 128, 0},   {32, 32, 1, 512, 0},
     {32, 16, 2, 512, 0}, {16, 16, 2, 512, 0}, {24, 24, 1, 512, 0},
     // coarse levels: one pixel per thread per half-sweep (fewer dependent loads in a row)
-    {8, 4, 2, 256, 0},   {8, 4, 2, 512, 0},   {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},   {16, 16, 1, 512, 0}, {8, 8, 6, 512, 0},
+    {8, 4, 2, 256, 0},   {8, 4, 2, 512, 0},   {8, 8, 3, 512, 0},   {8, 8, 2, 512, 0},   {16, 8, 2, 512, 0},
+    {16, 16, 1, 512, 0}, {8, 8, 6, 512, 0},
     // fine levels: larger tiles recompute a smaller share of halo pixels
     {64, 32, 1, 128, 0}, {48, 32, 1, 128, 0}, {48, 32, 1, 256, 0}, {64, 16, 1, 128, 0}, {40, 24, 1, 128, 0},
     {48, 24, 1, 128, 0}, {64, 24, 1, 256, 0}, {64, 24, 1, 128, 0}, {96, 24, 1, 256, 0}, {80, 24, 1, 256, 0},

@@ -258,8 +258,8 @@ bool prop_threads_ok(int threads);
 // Resident CTAs per SM of a tile or dataflow launch, in the variant it takes (n_iter: iterations per tile task).
 int prop_blocks_per_sm(int tw, int th, int n_iter, int threads, int cost, bool dataflow, bool listed);
 // Tile form (L.cluster == 0): queue_dev[i] = (problem index, tile index); counter_dev must be zero when the launch
-// starts; `grid` CTAs.  Dataflow form (L.dataflow = T): the same queue, taken T times (iteration-major).  Cluster form: problem i is probs_dev[i], `grid` = number of problems x L.cluster CTAs;
-// queue_dev and counter_dev are unused.
+// starts; `grid` CTAs.  Dataflow form (L.dataflow = T): the same queue, taken T times (iteration-major).  Cluster form:
+// problem i is probs_dev[i], `grid` = number of problems x L.cluster CTAs; queue_dev and counter_dev are unused.
 void launch_propagate(const PropProblem* probs_dev, const int2* queue_dev, int n_tiles, int* counter_dev, int grid,
                       const PropLaunch& L, cudaStream_t st);
 // Clusters of the cluster form that can be resident at once (0: this shape cannot be launched).
@@ -449,8 +449,9 @@ bool ctx_view(const ff_ctx* c, CtxView* out);
 bool ctx_owns_live_pyr(const ff_ctx* c, const ff_pyr* p);
 bool pyr_view(const ff_pyr* p, PyrView* out);
 // the launch configuration of a pass (level s, or its sub-scale grid s + 8k) of size w x h for the server and the
-// no-allocation entry point, which launch the tile form and (dataflow_ok) the dataflow form, never the cluster form; compact: an untuned
-// pass takes the configuration the no-allocation entry point's scratch is reckoned with instead of the fastest one
+// no-allocation entry point, which launch the tile form and (dataflow_ok) the dataflow form, never the cluster form;
+// compact: an untuned pass takes the configuration the no-allocation entry point's scratch is reckoned with instead of
+// the fastest one
 TileChoice ctx_level_choice(const ff_ctx* c, int level, int w, int h, int n_dirs, int64_t level_pix_all,
                             bool dataflow_ok, bool compact);
 // the context's error word of the bounded device waits, allocated on first use (null if that fails)

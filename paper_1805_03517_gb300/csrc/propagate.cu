@@ -348,8 +348,9 @@ __device__ __forceinline__ void halfsweep_direct(const SweepConst& K, const Tile
 // when the thread has nothing else to do; only a pixel that takes a neighbour's flow scores another one after it.  And
 // there is no index arithmetic.  Pass times (6 iterations, us) of the best tiles with / without, by pixels: WHT-SAD 96
 // 34 / 50, 1.5 k 54 / 58, 3.7 k 50 / 61, 10 k 68 / 78, 16 k 67 / 77, 25 k 82 / 94, 38 k 88 / 94, 42 k 102 / 98; Census
-// 33 / 43, 42 / 48, 45 / 50, 52 / 52, 57 / 53, 60 / 70, 72 / 74, 85 / 74.  (A pair of pixels per thread, one of each
-// colour and no thread idle, nor anything scored ahead: 90 instead of 61 at 3.7 k, spills included.)
+// 33 / 43, 42 / 48, 45 / 50, 52 / 52, 57 / 53, 60 / 70, 72 / 74, 85 / 74 (with two CTAs per SM; with the third 54 at 16 k).
+// (A pair of pixels per thread, one of each colour and no thread idle, nor anything scored ahead: 90 instead of 61 at 3.7 k,
+// spills included.)
 
 // Cost of the flow (fx, fy) of level pixel (X, Y) with descriptor a, INT_MAX if its target is outside the level.
 // (The arrays of predicated loads are zeroed, here and below: left uninitialised, they stay live around the loops and
@@ -474,38 +475,38 @@ __device__ __forceinline__ void propagate_tile_direct(const PropProblem& P, int 
     s_regions[0].set(G, w, h, kHaloPerIter * (n_iter - 1));
     if constexpr (RES) {
         propagate_tile_resident<C, DF>(K, G, P, smem, io, s_regions);
-        return;
-    }
-
-    for (int i = threadIdx.x; i < G.RW * G.RH; i += blockDim.x) {
-        int r = i / G.RW, c = i - r * G.RW;
-        size_t g = (size_t)(G.ly0 + r) * w + G.lx0 + c;
-        // flow and cost of the region (2 words per pixel) must fit the launch's dynamic shared memory
-        const bool ok = idx_ok(g_bounds, kBoundsTileRead, (long long)g, (long long)w * h) &&
-                        (!FF_DEBUG_BOUNDS || idx_ok(g_bounds, kBoundsTileSmem, 2 * G.RW * G.RH - 1, dyn_smem_bytes() / 4));
-        sflow[i] = !ok ? 0u : DF ? __ldcg(io.flow_in + g) : io.flow_in[g];
-        scost[i] = !ok ? 0 : DF ? __ldcg(io.cost_in + g) : io.cost_in[g];
-    }
-    __syncthreads();
-    for (int it = 0; it < n_iter; it++) {
-        const uint32_t k1 = iter_key(P, io.t0 + it);
-        const SweepRegions& S = s_regions[it & 1];
-        if (it + 1 < n_iter) s_regions[(it + 1) & 1].set(G, w, h, kHaloPerIter * (n_iter - 2 - it));
-        for (int j = 0; j < 8; j++) {
-            halfsweep_direct<C>(K, G, w, h, S.r[j], S.inv[j], sflow, scost, j, k1);
-            __syncthreads();
+    } else {
+        for (int i = threadIdx.x; i < G.RW * G.RH; i += blockDim.x) {
+            int r = i / G.RW, c = i - r * G.RW;
+            size_t g = (size_t)(G.ly0 + r) * w + G.lx0 + c;
+            // flow and cost of the region (2 words per pixel) must fit the launch's dynamic shared memory
+            const bool ok = idx_ok(g_bounds, kBoundsTileRead, (long long)g, (long long)w * h) &&
+                            (!FF_DEBUG_BOUNDS ||
+                             idx_ok(g_bounds, kBoundsTileSmem, 2 * G.RW * G.RH - 1, dyn_smem_bytes() / 4));
+            sflow[i] = !ok ? 0u : DF ? __ldcg(io.flow_in + g) : io.flow_in[g];
+            scost[i] = !ok ? 0 : DF ? __ldcg(io.cost_in + g) : io.cost_in[g];
         }
-    }
-    const int TW = G.x1 - G.x0;
-    for (int i = threadIdx.x; i < TW * (G.y1 - G.y0); i += blockDim.x) {
-        int r = i / TW, c = i - r * TW;
-        int sidx = (G.y0 + r - G.ly0) * G.RW + (G.x0 + c - G.lx0);
-        size_t g = (size_t)(G.y0 + r) * w + G.x0 + c;
-        if (!idx_ok(g_bounds, kBoundsTileWrite, (long long)g, (long long)w * h) ||
-            !idx_ok(g_bounds, kBoundsTileSmem, sidx, G.RW * G.RH))
-            continue;
-        io.flow_out[g] = sflow[sidx];
-        io.cost_out[g] = scost[sidx];
+        __syncthreads();
+        for (int it = 0; it < n_iter; it++) {
+            const uint32_t k1 = iter_key(P, io.t0 + it);
+            const SweepRegions& S = s_regions[it & 1];
+            if (it + 1 < n_iter) s_regions[(it + 1) & 1].set(G, w, h, kHaloPerIter * (n_iter - 2 - it));
+            for (int j = 0; j < 8; j++) {
+                halfsweep_direct<C>(K, G, w, h, S.r[j], S.inv[j], sflow, scost, j, k1);
+                __syncthreads();
+            }
+        }
+        const int TW = G.x1 - G.x0;
+        for (int i = threadIdx.x; i < TW * (G.y1 - G.y0); i += blockDim.x) {
+            int r = i / TW, c = i - r * TW;
+            int sidx = (G.y0 + r - G.ly0) * G.RW + (G.x0 + c - G.lx0);
+            size_t g = (size_t)(G.y0 + r) * w + G.x0 + c;
+            if (!idx_ok(g_bounds, kBoundsTileWrite, (long long)g, (long long)w * h) ||
+                !idx_ok(g_bounds, kBoundsTileSmem, sidx, G.RW * G.RH))
+                continue;
+            io.flow_out[g] = sflow[sidx];
+            io.cost_out[g] = scost[sidx];
+        }
     }
 }
 
@@ -723,8 +724,9 @@ bool prop_listed(int64_t pass_pixels, int64_t pass_tiles, int tw, int threads, i
            (T >= 10 || pass_tiles * threads >= (int64_t)n_sms * 1024) && (T >= 6 || pitch <= 64);
 }
 
-// The resident variant takes every tile it can (regions of at most one pixel per thread): in the same tiles it is never
-// slower (8x8 pixels and 256 threads: 57 instead of 73 us at level 4 of the 1242x375 pair, 72 instead of 80 at level 3).
+// The resident variant takes every tile it can (regions of at most one pixel per thread): in the same tiles it was not
+// slower in any of 4,320 passes of 1.2 k to 4.1 M pixels, both costs, 1, 3 and 6 iterations, 128 to 512 threads (8x8
+// pixels and 256 threads: 57 instead of 73 us at level 4 of the 1242x375 pair, 72 instead of 80 at level 3).
 bool prop_resident(int tw, int th, int n_iter, int threads) {
     const int H = kHaloPerIter * n_iter;
     return 2 * ((tw + 2 * H + 1) / 2) * (th + 2 * H) <= threads;
@@ -899,8 +901,8 @@ __device__ __forceinline__ void set_regions() {
 }
 
 // One tile of one problem: load the tile and its halo, run iteration io.t0 in shared memory, write the tile.  The state
-// was written by other CTAs of the running launch and is therefore read from L2.  Between the tasks of a pass the cost buffers hold state words; a pass starts from plain costs and its last
-// iteration leaves plain costs.  The head of the shared memory is set (tile_setup).
+// was written by other CTAs of the running launch and is therefore read from L2.  Between the tasks of a pass the cost
+// buffers hold state words; a pass starts from plain costs and its last iteration leaves plain costs.  The head of the shared memory is set (tile_setup).
 // With a counter, the CTA's next task is taken while this one is written, into *s_next.
 template <class C, int THREADS>
 __device__ __forceinline__ void propagate_tile_listed(const PropProblem& P, const TileLayout T, int* counter, int* s_next) {
@@ -998,8 +1000,8 @@ __device__ __forceinline__ void tile_setup(const PropProblem& P, int tile, const
 // queue[i] = (problem index, tile index in problem).
 // Instantiated for 128, 256 and 512 threads, per cost, direct and resident.
 // The Census kernels are held to the registers of three CTAs of 256 threads per SM (direct 78, resident 71; unbounded 92
-// and 85, two CTAs).  Direct: a 1920x1080 pair in 32x32 tiles 2.98 instead of 3.63 ms, a 1024x436 direction without
-// allocation 524 instead of 630 us.  Resident: 27.9 k pixels in 8x8 tiles (448 of them, on 304 CTAs two rounds) 57 us
+// and 85, two CTAs).  Direct: a 1920x1080 pair in 32x32 tiles 2.96 instead of 3.63 ms, a 1024x436 direction without
+// allocation 510 instead of 630 us.  Resident: 27.9 k pixels in 8x8 tiles (448 of them, on 304 CTAs two rounds) 57 us
 // instead of 90.
 template <int THREADS, class C, bool RES>
 __global__ __launch_bounds__(THREADS, (C::kSectors > 1 ? 512 : 768) / THREADS) void k_propagate(
@@ -1420,12 +1422,13 @@ void launch_propagate(const PropProblem* probs_dev, const int2* queue_dev, int n
     }
     const size_t smem = prop_launch_smem(L.tw, L.th, L.max_iter, L.listed != 0);
     const bool resident = prop_resident(L.tw, L.th, L.dataflow > 0 ? 1 : L.max_iter, L.threads);
+    const Variant v = L.listed ? kListed : resident ? kResident : kDirect;
     if (L.dataflow > 0)
-        launch_k(prop_df_kernel(L.threads, L.cost, L.listed ? kListed : resident ? kResident : kDirect), dim3(grid), dim3(L.threads), smem, st, probs_dev,
-                 queue_dev, n_tiles, counter_dev, L, tile_layout(L.tw, L.th));
+        launch_k(prop_df_kernel(L.threads, L.cost, v), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles,
+                 counter_dev, L, tile_layout(L.tw, L.th));
     else
-        launch_k(prop_kernel(L.threads, L.cost, resident), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev, n_tiles,
-                 counter_dev, L);
+        launch_k(prop_kernel(L.threads, L.cost, resident), dim3(grid), dim3(L.threads), smem, st, probs_dev, queue_dev,
+                 n_tiles, counter_dev, L);
 }
 
 }  // namespace ff
